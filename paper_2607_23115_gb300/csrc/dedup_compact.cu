@@ -37,6 +37,8 @@
 // k_small_call: the staged hash, then k_dedup's and k_pack's steps with a
 // grid of one block (every grid barrier a block barrier), so that the call
 // costs one launch and no kernel boundary.
+#include <algorithm>
+
 #include "gleam_internal.cuh"
 #include "staged_hash.cuh"
 
@@ -45,9 +47,6 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
-#ifndef GLEAM_COPY_STREAMING_STORES
-#define GLEAM_COPY_STREAMING_STORES 1
-#endif
 #ifndef GLEAM_COPY_VEC
 #define GLEAM_COPY_VEC 8
 #endif
@@ -78,75 +77,161 @@ constexpr uint32_t kSmallCmpWays = GLEAM_SMALL_CMP_WAYS;
 
 __device__ __forceinline__ uint32_t ldcg_u32(const uint32_t* p) { return __ldcg(p); }
 
-// Whole-warp byte equality of two full chunks of the payload.
-__device__ bool warp_equal(const uint8_t* x, const uint8_t* y, uint32_t len, bool vec) {
-  const uint32_t lane = threadIdx.x & 31;
-  bool diff = false;
-  uint32_t done = 0;
-  if (vec) {
-    const uint32_t nv = len >> 4;
-    const uint4* xv = reinterpret_cast<const uint4*>(x);
-    const uint4* yv = reinterpret_cast<const uint4*>(y);
-    for (uint32_t k0 = 0; k0 < nv; k0 += 128) {
-      uint4 u[4], w[4];
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const uint32_t k = k0 + r * 32 + lane;
-        if (k < nv) {
-          u[r] = __ldcs(xv + k);
-          w[r] = __ldcs(yv + k);
-        } else {
-          u[r] = make_uint4(0, 0, 0, 0);
-          w[r] = u[r];
-        }
-      }
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-        diff |= (u[r].x != w[r].x) | (u[r].y != w[r].y) | (u[r].z != w[r].z) | (u[r].w != w[r].w);
-      if (__any_sync(0xffffffffu, diff)) return false;
-    }
-    done = nv << 4;
+__device__ __forceinline__ bool differ16(uint4 x, uint4 y) {
+  return (x.x != y.x) | (x.y != y.y) | (x.z != y.z) | (x.w != y.w);
+}
+
+// Bytes [m, m + 16) of the 32 bytes a, b (m < 16).
+__device__ __forceinline__ uint4 shifted16(uint4 a, uint4 b, uint32_t m) {
+  uint32_t y0, y1, y2, y3, y4;
+  switch (m >> 2) {
+    case 0: y0 = a.x, y1 = a.y, y2 = a.z, y3 = a.w, y4 = b.x; break;
+    case 1: y0 = a.y, y1 = a.z, y2 = a.w, y3 = b.x, y4 = b.y; break;
+    case 2: y0 = a.z, y1 = a.w, y2 = b.x, y3 = b.y, y4 = b.z; break;
+    default: y0 = a.w, y1 = b.x, y2 = b.y, y3 = b.z, y4 = b.w; break;
   }
-  for (uint32_t k = done + lane; k < len; k += 32) diff |= (x[k] != y[k]);
+  const uint32_t r = (m & 3) * 8;
+  return make_uint4(__funnelshift_r(y0, y1, r), __funnelshift_r(y1, y2, r),
+                    __funnelshift_r(y2, y3, r), __funnelshift_r(y3, y4, r));
+}
+
+// The 16 bytes at p of any alignment, by the aligned 16-byte pieces that hold
+// them (both must be readable).
+__device__ __forceinline__ uint4 load16_any(const uint8_t* p) {
+  const uint32_t m = (uint32_t)((uintptr_t)p & 15);
+  const uint4* a = reinterpret_cast<const uint4*>(p - m);
+  if (m == 0) return __ldg(a);
+  return shifted16(__ldg(a), __ldg(a + 1), m);
+}
+
+// warp_equal for chunks of any alignment: 16 bytes at a time put together from
+// aligned pieces (load16_any) where those lie inside both chunks, the bytes at
+// either end one by one.  Out of line.
+__device__ __noinline__ bool warp_equal_any(const uint8_t* x, const uint8_t* y, uint32_t len) {
+  const uint32_t lane = threadIdx.x & 31;
+  const uint32_t k_lo = 1, k_hi = len < 32 ? 1u : (len - 16) >> 4;  // 16-byte steps [k_lo, k_hi)
+  bool diff = false;
+  for (uint32_t k0 = k_lo; k0 < k_hi; k0 += 64) {
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      const uint32_t k = k0 + r * 32 + lane;
+      if (k < k_hi) diff |= differ16(load16_any(x + 16ull * k), load16_any(y + 16ull * k));
+    }
+    if (__any_sync(0xffffffffu, diff)) return false;
+  }
+  for (uint32_t k = lane; k < min(len, 16u * k_lo); k += 32) diff |= (x[k] != y[k]);
+  for (uint32_t k = 16 * k_hi + lane; k < len; k += 32) diff |= (x[k] != y[k]);
   return !__any_sync(0xffffffffu, diff);
 }
 
-// Whole-warp copy of one chunk to the packed output and to its arena slot
-// (d2 == nullptr: to the packed output only).  The path of copies that cannot
-// be bulk copies (host or managed memory, unaligned addresses): out of line,
-// away from the code that every call runs.
-__device__ __noinline__ void warp_copy2(uint8_t* d1, uint8_t* d2, const uint8_t* s, uint32_t len, bool vec) {
+// Whole-warp byte equality of two chunks.
+__device__ bool warp_equal(const uint8_t* x, const uint8_t* y, uint32_t len) {
+  if ((((uintptr_t)x | (uintptr_t)y) & 15) != 0) return warp_equal_any(x, y, len);
   const uint32_t lane = threadIdx.x & 31;
-  uint32_t done = 0;
-  if (vec) {
-    const uint32_t nv = len >> 4;
-    const uint4* sv = reinterpret_cast<const uint4*>(s);
-    uint4* d1v = reinterpret_cast<uint4*>(d1);
-    uint4* d2v = reinterpret_cast<uint4*>(d2);
-    for (uint32_t k0 = 0; k0 < nv; k0 += 32 * kCopyVec) {
-      uint4 u[kCopyVec];
+  bool diff = false;
+  const uint32_t nv = len >> 4;
+  const uint4* xv = reinterpret_cast<const uint4*>(x);
+  const uint4* yv = reinterpret_cast<const uint4*>(y);
+  for (uint32_t k0 = 0; k0 < nv; k0 += 128) {
+    uint4 u[4], w[4];
 #pragma unroll
-      for (int r = 0; r < kCopyVec; ++r) {
-        const uint32_t k = k0 + r * 32 + lane;
-        if (k < nv) u[r] = __ldg(sv + k);
-      }
-#pragma unroll
-      for (int r = 0; r < kCopyVec; ++r) {
-        const uint32_t k = k0 + r * 32 + lane;
-        if (k < nv) {
-#if GLEAM_COPY_STREAMING_STORES
-          __stcs(d1v + k, u[r]);
-          if (d2) __stcs(d2v + k, u[r]);
-#else
-          d1v[k] = u[r];
-          if (d2) d2v[k] = u[r];
-#endif
-        }
+    for (int r = 0; r < 4; ++r) {
+      const uint32_t k = k0 + r * 32 + lane;
+      if (k < nv) {
+        u[r] = __ldcs(xv + k);
+        w[r] = __ldcs(yv + k);
+      } else {
+        u[r] = make_uint4(0, 0, 0, 0);
+        w[r] = u[r];
       }
     }
-    done = nv << 4;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) diff |= differ16(u[r], w[r]);
+    if (__any_sync(0xffffffffu, diff)) return false;
   }
-  for (uint32_t k = done + lane; k < len; k += 32) {
+  for (uint32_t k = (nv << 4) + lane; k < len; k += 32) diff |= (x[k] != y[k]);
+  return !__any_sync(0xffffffffu, diff);
+}
+
+// Whole-warp copy of len bytes at s to d1 and, if not null, to d2, in 16-byte
+// stores put together from the aligned 16-byte pieces of the payload that
+// hold them; s of any alignment, d1 and d2 of one alignment.  The bytes
+// before d1's first 16-byte boundary, and those at the payload's ends whose
+// pieces reach past it, go one by one.  Byte by byte throughout, the copies of
+// 26 MB of misses at 8-byte alignment took 1,035 us of a 1,489 us call (40
+// payloads, 260 MB, a tenth of their 16 KiB chunks changed); the second load
+// of each lane is its neighbour's first, so it comes from L1.
+__device__ __noinline__ void warp_copy_any(uint8_t* d1, uint8_t* d2, const uint8_t* s,
+                                           uint32_t len, const PayloadDesc& P) {
+  const uint8_t *lo = P.buf, *hi = P.buf + P.n;
+  const uint32_t lane = threadIdx.x & 31;
+  uint32_t head = (uint32_t)(0 - (uintptr_t)d1) & 15u;
+  const uint32_t m = (uint32_t)((uintptr_t)(s + head) & 15);
+  if (m && s + head - m < lo) head += 16;
+  uint32_t nv = len > head ? (len - head) >> 4 : 0u;
+  if (nv && m && s + head - m + 16ull * nv + 16 > hi) --nv;
+  const uint32_t tail = min(len, head) + (nv << 4);
+  for (uint32_t k0 = 0; k0 < nv; k0 += 128) {
+    uint4 u[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const uint32_t k = k0 + r * 32 + lane;
+      if (k < nv) u[r] = load16_any(s + head + 16ull * k);
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const uint32_t k = k0 + r * 32 + lane;
+      if (k < nv) {
+        __stcs(reinterpret_cast<uint4*>(d1 + head) + k, u[r]);
+        if (d2) __stcs(reinterpret_cast<uint4*>(d2 + head) + k, u[r]);
+      }
+    }
+  }
+  auto bytes = [&](uint32_t k0, uint32_t k1) {
+    for (uint32_t k = k0 + lane; k < k1; k += 32) {
+      const uint8_t b = s[k];
+      d1[k] = b;
+      if (d2) d2[k] = b;
+    }
+  };
+  bytes(0, min(len, head));
+  bytes(tail, len);
+}
+
+// Whole-warp copy of a piece of a chunk to the packed output and to its arena
+// slot (d2 == nullptr: to the packed output only).  The path of copies that cannot
+// be bulk copies (host or managed memory, unaligned addresses): out of line,
+// away from the code that every call runs.  P: the piece's payload.
+__device__ __noinline__ void warp_copy2(uint8_t* d1, uint8_t* d2, const uint8_t* s, uint32_t len,
+                                        const PayloadDesc& P) {
+  if ((((uintptr_t)d1 | (uintptr_t)d2 | (uintptr_t)s) & 15) != 0) {
+    const bool apart = d2 && (((uintptr_t)d1 ^ (uintptr_t)d2) & 15) != 0;
+    warp_copy_any(d1, apart ? nullptr : d2, s, len, P);
+    if (apart) warp_copy_any(d2, nullptr, s, len, P);
+    return;
+  }
+  const uint32_t lane = threadIdx.x & 31;
+  const uint32_t nv = len >> 4;
+  const uint4* sv = reinterpret_cast<const uint4*>(s);
+  uint4* d1v = reinterpret_cast<uint4*>(d1);
+  uint4* d2v = reinterpret_cast<uint4*>(d2);
+  for (uint32_t k0 = 0; k0 < nv; k0 += 32 * kCopyVec) {
+    uint4 u[kCopyVec];
+#pragma unroll
+    for (int r = 0; r < kCopyVec; ++r) {
+      const uint32_t k = k0 + r * 32 + lane;
+      if (k < nv) u[r] = __ldg(sv + k);
+    }
+#pragma unroll
+    for (int r = 0; r < kCopyVec; ++r) {
+      const uint32_t k = k0 + r * 32 + lane;
+      if (k < nv) {
+        __stcs(d1v + k, u[r]);
+        if (d2) __stcs(d2v + k, u[r]);
+      }
+    }
+  }
+  for (uint32_t k = (nv << 4) + lane; k < len; k += 32) {
     const uint8_t b = s[k];
     d1[k] = b;
     if (d2) d2[k] = b;
@@ -182,7 +267,7 @@ struct PackMeta {
 // a multiple of 128 bytes so that every warp's buffers start 128-byte aligned
 constexpr uint32_t kPackWarpBytes =
     (kPackBufs * kPackPiece + 64 + 32 * (uint32_t)sizeof(PackMeta) + 127) & ~127u;
-constexpr uint32_t kPackSmem = GLEAM_PACK_BULK ? kWarps * kPackWarpBytes : 0;
+constexpr uint32_t kPackSmem = kWarps * kPackWarpBytes;
 
 __device__ __forceinline__ void mbar_init(uint32_t bar) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
@@ -930,8 +1015,7 @@ __device__ __forceinline__ void resolve_rank(const DedupArgs& a, uint32_t G, uin
         const uint8_t* x = reinterpret_cast<const uint8_t*>(__shfl_sync(0xffffffffu, xs, j));
         const uint8_t* y = reinterpret_cast<const uint8_t*>(__shfl_sync(0xffffffffu, ys, j));
         const uint32_t len = __shfl_sync(0xffffffffu, ln, j);
-        const bool vec = (((uintptr_t)x | (uintptr_t)y) & 15) == 0;
-        settle(j, warp_equal(x, y, len, vec));
+        settle(j, warp_equal(x, y, len));
       }
     }
     if (G == 1) {  // the block's own count, without the round trip to the counter
@@ -1224,6 +1308,9 @@ __device__ __forceinline__ void finish_call(const DedupArgs& a, uint32_t G,
 // rank copied by whole warps to the packed output and its arena slot and
 // inserted into the index; the last block publishes the counters and results
 // and leaves the per-call state zeroed.  Nothing is written after an error.
+// kPlain: the misses are copied by whole warps (DedupArgs::plain_copy), a
+// variant of its own so that the bulk copies' kernels carry none of its code.
+template <bool kPlain>
 __device__ __forceinline__ void pack_publish(const DedupArgs& a, uint32_t G, uint32_t bid,
                                              uint8_t* pack_smem) {
   __shared__ unsigned long long red64[kWarps];
@@ -1248,19 +1335,20 @@ __device__ __forceinline__ void pack_publish(const DedupArgs& a, uint32_t G, uin
   const unsigned long long total = s_total;
   const unsigned long long evict = s_evict;
   const bool ok = s_err == 0;
-#if GLEAM_PACK_BULK
-  const uint32_t wbase = (uint32_t)__cvta_generic_to_shared(pack_smem) + w * kPackWarpBytes;
+  const uint32_t wbase =
+      kPlain ? 0u : (uint32_t)__cvta_generic_to_shared(pack_smem) + w * kPackWarpBytes;
   const uint32_t bufs = wbase, bars = wbase + kPackBufs * kPackPiece;
   PackMeta* meta = reinterpret_cast<PackMeta*>(pack_smem + w * kPackWarpBytes +
                                                kPackBufs * kPackPiece + 64);
   PackRing ring{0u, 0u, 0u};
-  if (lane == 0) {
-    for (uint32_t b = 0; b < kPackBufs; ++b) mbar_init(bars + 8 * b);
-    mbar_fence_init();
+  if constexpr (!kPlain) {
+    if (lane == 0) {
+      for (uint32_t b = 0; b < kPackBufs; ++b) mbar_init(bars + 8 * b);
+      mbar_fence_init();
+    }
+    __syncwarp();
   }
-  __syncwarp();
   bool bulk_failed = false;
-#endif
   // slot of the stored miss of stored rank sr: the evicted slots in ascending
   // order, then never-used slots
   auto slot_of = [&](uint32_t sr) -> unsigned long long {
@@ -1422,13 +1510,14 @@ __device__ __forceinline__ void pack_publish(const DedupArgs& a, uint32_t G, uin
       uint32_t bytes = 0;
       bool copy = false;
       unsigned long long src = 0, d1 = 0, d2 = 0;
+      uint32_t pp = 0;
       if (pc < shi) {
         const unsigned long long r = pc / ppc;
         const uint32_t off = (uint32_t)(pc - r * ppc) * kPackPiece;
         const uint32_t gg = ch.order[r];
         const uint32_t ln = ch.len[gg];
         if (off < ln) {
-          const uint32_t pp = ch.pidx[gg];
+          pp = ch.pidx[gg];
           const PayloadDesc& P = desc(a, pp);
           bytes = min(kPackPiece, ln - off);
           src = ch.src[gg] + off;
@@ -1443,10 +1532,7 @@ __device__ __forceinline__ void pack_publish(const DedupArgs& a, uint32_t G, uin
       }
       const unsigned cmask = __ballot_sync(0xffffffffu, copy);  // lanes whose piece is copied
       const uint32_t m = __popc(cmask);
-#if GLEAM_PACK_BULK
-      const bool bulk =
-          !a.plain_copy && __all_sync(0xffffffffu, !copy || ((src | d1 | d2) & 15) == 0);
-      if (bulk) {
+      if constexpr (!kPlain) {
         if (copy) meta[__popc(cmask & ((1u << lane) - 1u))] = PackMeta{src, d1, d2, bytes, 0u};
         __syncwarp();
         if (lane == 0 && m && !bulk_failed &&
@@ -1464,16 +1550,16 @@ __device__ __forceinline__ void pack_publish(const DedupArgs& a, uint32_t G, uin
           }
         }
         __syncwarp();
-      } else
-#endif
-      for (unsigned todo = cmask; todo; todo &= todo - 1) {
+      }
+      for (unsigned todo = kPlain ? cmask : 0u; todo; todo &= todo - 1) {
         const int j = __ffs(todo) - 1;
         const unsigned long long sj = __shfl_sync(0xffffffffu, src, j);
         const unsigned long long xj = __shfl_sync(0xffffffffu, d1, j);
         const unsigned long long yj = __shfl_sync(0xffffffffu, d2, j);
         const uint32_t lj = __shfl_sync(0xffffffffu, bytes, j);
         warp_copy2(reinterpret_cast<uint8_t*>(xj), reinterpret_cast<uint8_t*>(yj),
-                   reinterpret_cast<const uint8_t*>(sj), lj, ((sj | xj | yj) & 15) == 0);
+                   reinterpret_cast<const uint8_t*>(sj), lj,
+                   desc(a, __shfl_sync(0xffffffffu, pp, j)));
       }
       if (grab) {
         const unsigned long long v = __shfl_sync(0xffffffffu, next, 0);
@@ -1506,9 +1592,7 @@ __device__ __forceinline__ void pack_publish(const DedupArgs& a, uint32_t G, uin
           !index_insert(a.hints, a.index_mask, ch.hint[gg], (uint32_t)slot, ln))
         atomicCAS(&a.ctl->err, 0, (int)GLEAM_ERR_INTERNAL);
     }
-#if GLEAM_PACK_BULK
-    if (lane == 0) bulk_wait_all<0>();  // every piece written before the block ends
-#endif
+    if (!kPlain && lane == 0) bulk_wait_all<0>();  // every piece written before the block ends
     n_hc = block_sum<unsigned long long>(n_hc, red64);
     n_hi = block_sum<unsigned long long>(n_hi, red64);
     n_rej = block_sum<unsigned long long>(n_rej, red64);
@@ -1554,7 +1638,6 @@ __device__ __forceinline__ void pack_publish(const DedupArgs& a, uint32_t G, uin
 // the most of them as the call's tail).  Otherwise the general algorithm
 // takes over: the minima are posted and resolve_rank and pack_publish run on
 // the same grid.
-constexpr uint32_t kResolvePackSmem = kPackSmem;
 
 
 // Bit k of the result: byte k of w (k < 4) is not kHit0.
@@ -1598,6 +1681,7 @@ __device__ __forceinline__ void count_not_hit(const uint8_t* status, uint32_t N,
 // the common path's code stays compact (the kernel runs once per call, on SMs
 // whose instruction caches are cold).  Every thread of every block calls it;
 // mine: this thread holds a chunk of a group (entry e, group key and length).
+template <bool kPlain>
 __device__ __noinline__ void resolve_pack_general(const DedupArgs& a, uint32_t G, uint32_t bid,
                                                   uint8_t* smem, bool ok, bool pre, bool mine,
                                                   uint32_t e, unsigned long long key,
@@ -1620,9 +1704,10 @@ __device__ __noinline__ void resolve_pack_general(const DedupArgs& a, uint32_t G
   ok = grid_barrier(a.ctl, G, a.wait_ns, false);
   resolve_rank(a, G, bid, true, ok);
   grid_barrier(a.ctl, G, a.wait_ns, false);
-  pack_publish(a, G, bid, smem);
+  pack_publish<kPlain>(a, G, bid, smem);
 }
 
+template <bool kPlain>
 __device__ __forceinline__ void resolve_pack_fast(const DedupArgs& a, uint32_t G, uint32_t bid,
                                                   uint8_t* smem) {
   __shared__ unsigned long long red64[kWarps];
@@ -1722,7 +1807,7 @@ __device__ __forceinline__ void resolve_pack_fast(const DedupArgs& a, uint32_t G
   }
 
   if (s_shared) {
-    resolve_pack_general(a, G, bid, smem, ok, pre, valid && st != kHit0 && st != kUncached, e,
+    resolve_pack_general<kPlain>(a, G, bid, smem, ok, pre, valid && st != kHit0 && st != kUncached, e,
                          key, len, g);
     return;
   }
@@ -1819,18 +1904,19 @@ __device__ __forceinline__ void resolve_pack_fast(const DedupArgs& a, uint32_t G
     const unsigned long long ppc = (a.C + kPackPiece - 1) / kPackPiece;
     const unsigned long long npieces = total * ppc;
     const unsigned long long plo = npieces * gw / nw, phi = npieces * (gw + 1) / nw;
-#if GLEAM_PACK_BULK
-    const uint32_t wbase = (uint32_t)__cvta_generic_to_shared(smem) + w * kPackWarpBytes;
+    const uint32_t wbase =
+        kPlain ? 0u : (uint32_t)__cvta_generic_to_shared(smem) + w * kPackWarpBytes;
     const uint32_t bufs = wbase, bars = wbase + kPackBufs * kPackPiece;
     PackMeta* meta = reinterpret_cast<PackMeta*>(smem + w * kPackWarpBytes + kPackBufs * kPackPiece + 64);
     PackRing ring{0u, 0u, 0u};
     bool bulk_failed = false;
-    if (lane == 0) {
-      for (uint32_t b = 0; b < kPackBufs; ++b) mbar_init(bars + 8 * b);
-      mbar_fence_init();
+    if constexpr (!kPlain) {
+      if (lane == 0) {
+        for (uint32_t b = 0; b < kPackBufs; ++b) mbar_init(bars + 8 * b);
+        mbar_fence_init();
+      }
+      __syncwarp();
     }
-    __syncwarp();
-#endif
     // pieces [lo, hi) of the call, 32 at a time
     auto copy_range = [&](unsigned long long lo, unsigned long long hi) {
       for (unsigned long long base = lo; base < hi; base += 32) {
@@ -1857,10 +1943,7 @@ __device__ __forceinline__ void resolve_pack_fast(const DedupArgs& a, uint32_t G
           }
         }
         const unsigned cmask = __ballot_sync(0xffffffffu, copy);
-#if GLEAM_PACK_BULK
-        const bool bulk =
-            !a.plain_copy && __all_sync(0xffffffffu, !copy || ((src | d1 | d2) & 15) == 0);
-        if (bulk) {
+        if constexpr (!kPlain) {
           if (copy) meta[__popc(cmask & ((1u << lane) - 1u))] = PackMeta{src, d1, d2, bytes, 0u};
           __syncwarp();
           if (lane == 0 && cmask && !bulk_failed &&
@@ -1878,16 +1961,15 @@ __device__ __forceinline__ void resolve_pack_fast(const DedupArgs& a, uint32_t G
             }
           }
           __syncwarp();
-        } else
-#endif
-        for (unsigned todo = cmask; todo; todo &= todo - 1) {
+        }
+        for (unsigned todo = kPlain ? cmask : 0u; todo; todo &= todo - 1) {
           const int j = __ffs(todo) - 1;
           const unsigned long long sj = __shfl_sync(0xffffffffu, src, j);
           const unsigned long long xj = __shfl_sync(0xffffffffu, d1, j);
           const unsigned long long yj = __shfl_sync(0xffffffffu, d2, j);
           const uint32_t lj = __shfl_sync(0xffffffffu, bytes, j);
           warp_copy2(reinterpret_cast<uint8_t*>(xj), reinterpret_cast<uint8_t*>(yj),
-                     reinterpret_cast<const uint8_t*>(sj), lj, ((sj | xj | yj) & 15) == 0);
+                     reinterpret_cast<const uint8_t*>(sj), lj, P);
         }
       }
     };
@@ -1909,7 +1991,7 @@ __device__ __forceinline__ void resolve_pack_fast(const DedupArgs& a, uint32_t G
 #if GLEAM_CHAIN_PREFETCH
       // the warp's source pieces start their way into L2 at once (up to 32),
       // so that the copies below wait for L2 rather than HBM
-      if (plo + lane < phi && !a.plain_copy) {
+      if (plo + lane < phi && !a.far) {
         const unsigned long long pc = plo + lane, rr = pc / ppc;
         const uint32_t off = (uint32_t)(pc - rr * ppc) * kPackPiece;
         const uint32_t gg = __ldcg(&ch.order[rr]);
@@ -1934,9 +2016,7 @@ __device__ __forceinline__ void resolve_pack_fast(const DedupArgs& a, uint32_t G
         atomicCAS(&a.ctl->err, 0, (int)GLEAM_ERR_INTERNAL);
       if (e != 0xFFFFFFFFu) a.tbl[e] = CallEntry{0u, 0u};  // owner and the claim's tag
     }
-#if GLEAM_PACK_BULK
-    if (lane == 0) bulk_wait_all<0>();  // every piece written before the block ends
-#endif
+    if (!kPlain && lane == 0) bulk_wait_all<0>();  // every piece written before the block ends
   }
   n_hc = block_sum<unsigned long long>(n_hc, red64);
   n_rej = block_sum<unsigned long long>(n_rej, red64);
@@ -1972,11 +2052,12 @@ __device__ __forceinline__ void resolve_pack_fast(const DedupArgs& a, uint32_t G
   finish_call(a, G, slots0, total, stotal, 0ull, 0ull, s_sum);
 }
 
+template <bool kPlain>
 __global__ void __launch_bounds__(kThreads) k_resolve_pack(DedupArgs a) {
   extern __shared__ __align__(128) uint8_t rp_smem[];
   pdl_trigger();
   pdl_wait();
-  resolve_pack_fast(a, gridDim.x, blockIdx.x, rp_smem);
+  resolve_pack_fast<kPlain>(a, gridDim.x, blockIdx.x, rp_smem);
 }
 
 #ifndef GLEAM_DEDUP_MINBLOCKS
@@ -1990,11 +2071,12 @@ __global__ void __launch_bounds__(kThreads, GLEAM_DEDUP_MINBLOCKS) k_dedup(Dedup
   resolve_rank(a, gridDim.x, blockIdx.x);
 }
 
+template <bool kPlain>
 __global__ void GLEAM_PACK_BOUNDS k_pack(DedupArgs a) {
   extern __shared__ __align__(128) uint8_t pack_smem[];
   pdl_trigger();
   pdl_wait();
-  pack_publish(a, gridDim.x, blockIdx.x, pack_smem);
+  pack_publish<kPlain>(a, gridDim.x, blockIdx.x, pack_smem);
 }
 
 // A whole small call in one block: the staged hash of its chunks (kThreads / 4
@@ -2009,40 +2091,47 @@ constexpr uint32_t kSmallSmem = kSmallHashSmem > kPackSmem ? kSmallHashSmem : kP
 // k_dedup's and k_pack's steps on a grid of one block (several payloads, LRU,
 // a class table, or more chunks than threads): out of line, so that the small
 // kernel's common path stays compact.
+template <bool kPlain>
 __device__ __noinline__ void small_call_general(const DedupArgs& a, uint8_t* smem) {
   resolve_rank(a, 1, 0);
   __syncthreads();
-  pack_publish(a, 1, 0, smem);
+  pack_publish<kPlain>(a, 1, 0, smem);
 }
 
-template <bool kAhead, bool kPrefixAsync>
-__global__ void __launch_bounds__(kThreads) k_small_call(HashArgs h, DedupArgs a) {
+//
+// One block per SM at least: without saying so the compiler keeps to 102
+// registers and waits for more loads one by one (a 6 KB call of hits, back to
+// back: 14.8 us against 13.9).
+template <bool kAhead, bool kPrefixAsync, bool kMis, bool kPlain>
+__global__ void __launch_bounds__(kThreads, 1) k_small_call(HashArgs h, DedupArgs a) {
   extern __shared__ __align__(128) uint8_t small_smem[];
   pdl_trigger();
   if (!h.wait_late) pdl_wait();  // else in staged_range, before the first probe
-  // Device-resident payloads (16-byte aligned here) are prefetched into L2 at
-  // once, lane p taking payload p in 16 KiB pieces, so that the hash stages
-  // wait for L2 rather than HBM.
+  // Device-resident payloads are prefetched into L2 at once, lane p taking the
+  // whole 16-byte pieces of payload p, 16 KiB at a time, so that the hash
+  // stages wait for L2 rather than HBM.
   constexpr uint32_t kPiece = 16u << 10;
-  if (!a.plain_copy && a.count <= 32 && threadIdx.x < a.count) {
+  if (!a.far && a.count <= 32 && threadIdx.x < a.count) {
     const PayloadDesc& P = desc(a, threadIdx.x);
-    const unsigned long long nb = P.n & ~15ull;
+    const uint8_t* b0 = P.buf + (kMis ? (0 - (uintptr_t)P.buf) & 15 : 0);
+    const unsigned long long skip = b0 - P.buf;
+    const unsigned long long nb = P.n > skip ? (P.n - skip) & ~15ull : 0ull;
     for (unsigned long long off = 0; off < nb; off += kPiece)
-      prefetch_l2(P.buf + off, (uint32_t)min((unsigned long long)kPiece, nb - off));
+      prefetch_l2(b0 + off, (uint32_t)min((unsigned long long)kPiece, nb - off));
   }
   const unsigned long long nvb = (h.Ntot * 4 + kThreads - 1) / kThreads;
   for (unsigned long long vb = 0; vb < nvb; ++vb) {
     __syncthreads();  // the previous range's groups are done with the shared memory
-    staged_range<true, kAhead, true, kPrefixAsync>(h, vb, small_smem);
+    staged_range<true, kAhead, true, kPrefixAsync, kStage, kMis>(h, vb, small_smem);
   }
   __syncthreads();  // every chunk's probe outcome written (and its stage copies landed)
   if (a.count == 1 && !a.lru && !a.classes && a.Ntot <= (unsigned long long)kThreads) {
     // one payload of at most one chunk per thread: the one-launch path's
     // steps, which for a call without duplicates rank the misses by a block
     // scan (no LRU: they stamp no last use)
-    resolve_pack_fast(a, 1, 0, small_smem);
+    resolve_pack_fast<kPlain>(a, 1, 0, small_smem);
   } else {
-    small_call_general(a, small_smem);
+    small_call_general<kPlain>(a, small_smem);
   }
 }
 
@@ -2062,8 +2151,7 @@ __global__ void __launch_bounds__(kThreads) k_block_check(BlockCheckArgs a) {
       if (off <= a.block_bytes && len <= a.block_bytes - off) {
         const uint8_t* x = a.block + off;
         const uint8_t* y = a.arena + (unsigned long long)slot * a.C;
-        const bool vec = (((uintptr_t)x | (uintptr_t)y) & 15) == 0;
-        differs = !warp_equal(x, y, len, vec);
+        differs = !warp_equal(x, y, len);
       }
     }
     if (lane == 0) {
@@ -2147,30 +2235,28 @@ int dedup_threads() { return kThreads; }
 
 int dedup_chunks_per_block() { return GLEAM_DEDUP_CHUNKS_PER_BLOCK; }
 
-// Co-resident blocks per SM of the pack kernel.
-int pack_blocks_per_sm() {
+// Dynamic shared memory of a pack or one-launch resolve variant: the bulk
+// copies' buffers.
+constexpr uint32_t pack_smem_bytes(bool plain) { return plain ? 0u : kPackSmem; }
+
+template <typename K>
+int blocks_per_sm(K kern, uint32_t smem) {
   int nb = 0;
-  if (kPackSmem > 48 * 1024 &&
-      cudaFuncSetAttribute((const void*)k_pack, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           kPackSmem) != cudaSuccess)
-    return 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_pack, kThreads, kPackSmem) !=
-      cudaSuccess)
+  if (cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
+          cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, kThreads, smem) != cudaSuccess)
     return 0;
   return nb;
 }
 
+// Co-resident blocks per SM of the pack kernel.
+int pack_blocks_per_sm() { return blocks_per_sm(k_pack<false>, pack_smem_bytes(false)); }
+
 // Co-resident blocks per SM of the one-launch resolve + pack kernel (its grid
 // barriers need every block of the grid resident at once).
 int resolve_pack_blocks_per_sm() {
-  int nb = 0;
-  if (cudaFuncSetAttribute((const void*)k_resolve_pack, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           kResolvePackSmem) != cudaSuccess)
-    return 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_resolve_pack, kThreads,
-                                                    kResolvePackSmem) != cudaSuccess)
-    return 0;
-  return nb;
+  return std::min(blocks_per_sm(k_resolve_pack<false>, pack_smem_bytes(false)),
+                  blocks_per_sm(k_resolve_pack<true>, pack_smem_bytes(true)));
 }
 
 // Co-resident blocks per SM for the cooperative launch (capped).
@@ -2191,34 +2277,44 @@ cudaError_t launch_dedup(const DedupArgs& a, int grid, int pack_grid, cudaStream
     e = cudaLaunchCooperativeKernel((void*)k_dedup, dim3(grid), dim3(kThreads), args, 0, s);
   }
   if (e != cudaSuccess) return e;
-  if (kPackSmem > 48 * 1024)
-    cudaFuncSetAttribute((const void*)k_pack, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         kPackSmem);
-  return launch_kernel(k_pack, dim3(pack_grid), dim3(kThreads), kPackSmem, s, pdl, a);
+  auto pack = a.plain_copy ? k_pack<true> : k_pack<false>;
+  const uint32_t smem = pack_smem_bytes(a.plain_copy);
+  cudaFuncSetAttribute((const void*)pack, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  return launch_kernel(pack, dim3(pack_grid), dim3(kThreads), smem, s, pdl, a);
 }
 
 cudaError_t launch_resolve_pack(const DedupArgs& a, int grid, cudaStream_t s) {
-  cudaFuncSetAttribute((const void*)k_resolve_pack, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       kResolvePackSmem);
-  return launch_kernel(k_resolve_pack, dim3(grid), dim3(kThreads), kResolvePackSmem, s, true, a);
+  auto kern = a.plain_copy ? k_resolve_pack<true> : k_resolve_pack<false>;
+  const uint32_t smem = pack_smem_bytes(a.plain_copy);
+  cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  return launch_kernel(kern, dim3(grid), dim3(kThreads), smem, s, true, a);
 }
 
 uint32_t small_call_groups() { return kSmallGroups; }
 
-template <bool kAhead, bool kPrefixAsync>
+template <bool kAhead, bool kPrefixAsync, bool kMis, bool kPlain>
 cudaError_t launch_small(const HashArgs& h, const DedupArgs& a, cudaStream_t s, bool pdl) {
-  cudaFuncSetAttribute((const void*)k_small_call<kAhead, kPrefixAsync>,
-                       cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallSmem);
-  return launch_kernel(k_small_call<kAhead, kPrefixAsync>, dim3(1), dim3(kThreads), kSmallSmem, s,
-                       pdl, h, a);
+  auto kern = k_small_call<kAhead, kPrefixAsync, kMis, kPlain>;
+  cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallSmem);
+  return launch_kernel(kern, dim3(1), dim3(kThreads), kSmallSmem, s, pdl, h, a);
 }
 
-cudaError_t launch_small_call(const HashArgs& h, const DedupArgs& a, cudaStream_t s, bool pdl) {
-  if (h.C <= kPrefixAsyncMaxChunk)
-    return h.spec_mode ? launch_small<true, true>(h, a, s, pdl)
-                       : launch_small<false, true>(h, a, s, pdl);
-  return h.spec_mode ? launch_small<true, false>(h, a, s, pdl)
-                     : launch_small<false, false>(h, a, s, pdl);
+template <bool kPrefixAsync>
+cudaError_t launch_small(const HashArgs& h, const DedupArgs& a, bool aligned, cudaStream_t s,
+                         bool pdl) {
+  // unaligned payloads: no write-through (its 16-byte stores want aligned ones)
+  if (!aligned) return launch_small<false, kPrefixAsync, true, true>(h, a, s, pdl);
+  if (a.plain_copy)
+    return h.spec_mode ? launch_small<true, kPrefixAsync, false, true>(h, a, s, pdl)
+                       : launch_small<false, kPrefixAsync, false, true>(h, a, s, pdl);
+  return h.spec_mode ? launch_small<true, kPrefixAsync, false, false>(h, a, s, pdl)
+                     : launch_small<false, kPrefixAsync, false, false>(h, a, s, pdl);
+}
+
+cudaError_t launch_small_call(const HashArgs& h, const DedupArgs& a, bool aligned,
+                              cudaStream_t s, bool pdl) {
+  return h.C <= kPrefixAsyncMaxChunk ? launch_small<true>(h, a, aligned, s, pdl)
+                                     : launch_small<false>(h, a, aligned, s, pdl);
 }
 
 cudaError_t launch_block_check(const BlockCheckArgs& a, cudaStream_t s) {

@@ -463,13 +463,12 @@ constexpr uint64_t kSmallMaxBytes = 256ull << 10;
 // Whether a call runs as one single-block kernel instead of three launches:
 // few chunks and bytes (one block then hashes them about as fast as a grid
 // does, and a grid of one drops the kernel boundaries and every grid-wide
-// round trip: a 64 KiB call takes 24 us instead of 32), payloads the staged
-// hash can read, 64-bit or KEY16 keys, and no possible eviction (an evicting
-// call scans the whole index, which wants the full grid).
-bool small_call(const gleam_cache* c, bool aligned, uint64_t Ntot, uint64_t nbytes,
-                int skip_block) {
-  return Ntot > 0 && Ntot <= c->small_max_chunks && nbytes <= kSmallMaxBytes && aligned &&
-         (c->C % 32 == 0 || Ntot == 1) && !(c->flags & GLEAM_PAPER_IDS) && skip_block < 0 &&
+// round trip: a 64 KiB call takes 24 us instead of 32), 64-bit or KEY16 keys,
+// and no possible eviction (an evicting call scans the whole index, which
+// wants the full grid).
+bool small_call(const gleam_cache* c, uint64_t Ntot, uint64_t nbytes, int skip_block) {
+  return Ntot > 0 && Ntot <= c->small_max_chunks && nbytes <= kSmallMaxBytes &&
+         !(c->flags & GLEAM_PAPER_IDS) && skip_block < 0 &&
          (!(c->flags & GLEAM_EVICT_LRU) || c->slots_bound + Ntot <= c->nslots);
 }
 
@@ -571,7 +570,7 @@ unsigned long long stream_id(cudaStream_t s) {
 }
 
 // The write-through fields of a call's kernel arguments.  It needs the staged
-// hash (16-byte-aligned payloads, C a multiple of 32), 16-byte-aligned packed
+// hash on 16-byte-aligned payloads (C is a multiple of 32), 16-byte-aligned packed
 // buffers (device or page-locked host memory), and 64-bit or KEY16 keys.  In the automatic
 // mode the host launches the write-through variant of the hash kernel when
 // the page-locked copy of the device state says it is on (as of the last call
@@ -582,7 +581,7 @@ void set_spec(gleam_cache* c, HashArgs* h, DedupArgs* d, bool eligible) {
   d->spec_active = 0;
   d->spec_state = nullptr;
   d->spec_mirror = nullptr;
-  if (!eligible || c->C % 32 != 0 || (c->flags & GLEAM_PAPER_IDS) || c->spec_hook == 2) return;
+  if (!eligible || (c->flags & GLEAM_PAPER_IDS) || c->spec_hook == 2) return;
   const bool on = c->spec_hook == 1 || *reinterpret_cast<volatile uint32_t*>(c->spec_mirror);
   h->spec_mode = on ? 1u : 0u;
   h->arena_w = c->arena;
@@ -701,7 +700,8 @@ int enqueue(gleam_cache* c, const gleam_payload_t* payloads, uint64_t count,
   d.key16 = (c->flags & GLEAM_KEY16) ? 1u : 0u;
   d.classes = d.key16 && !d.paper ? 1u : 0u;
   d.cls_tbl = c->cls_tbl;
-  d.plain_copy = (host_payloads || chk.saw_managed()) ? 1u : 0u;
+  d.far = (host_payloads || chk.saw_managed()) ? 1u : 0u;
+  d.plain_copy = (d.far || !aligned || !packed_aligned) ? 1u : 0u;
   d.tbl = c->tbl;
   d.tbl_mask = tcap - 1;
   d.bcount = c->bcount;
@@ -719,7 +719,7 @@ int enqueue(gleam_cache* c, const gleam_payload_t* payloads, uint64_t count,
     grid = std::max(grid, std::min(2, c->coop_max_blocks));  // someone must be left waiting
     if (d.skip_block >= grid) d.skip_block = grid - 1;
   }
-  const bool fused = small_call(c, aligned, Ntot, nbytes, d.skip_block);
+  const bool fused = small_call(c, Ntot, nbytes, d.skip_block);
   const bool chain = chain_call(c, Ntot, nbytes, d.skip_block);
   // overlapping calls: the staged hash kernels fingerprint before they wait
   // (others ignore the field and wait first); the write-through stays off, as
@@ -752,7 +752,7 @@ int enqueue(gleam_cache* c, const gleam_payload_t* payloads, uint64_t count,
   // (Llama-3-8B, one call per tensor: +1%, four layers of it: +3%), where an
   // equal share per warp suits the one-block-per-SM grid of a call on its own
   if (one_launch && rp_grid > 1 && (c->flags & GLEAM_OVERLAP_CALLS)) d.copy_grab = kOverlapCopyGrab;
-  if (one_launch && rp_grid > 1 && hash_is_staged(h, aligned)) {
+  if (one_launch && rp_grid > 1 && hash_is_staged(h)) {
     h.claim_tbl = d.tbl;
     h.claim_mask = d.tbl_mask;
     d.pre_claimed = 1u;
@@ -770,7 +770,7 @@ int enqueue(gleam_cache* c, const gleam_payload_t* payloads, uint64_t count,
     cudaEventRecord(ev[0], s);
   }
   if (fused) {  // one kernel: all of its time is phase 0
-    if ((rc = cuda_err(launch_small_call(h, d, s, chain))) != GLEAM_OK) return rc;
+    if ((rc = cuda_err(launch_small_call(h, d, aligned, s, chain))) != GLEAM_OK) return rc;
     if (ev[1]) cudaEventRecord(ev[1], s);
   } else {
     if ((rc = cuda_err(launch_hash(h, aligned, s, chain))) != GLEAM_OK) return rc;
@@ -1496,7 +1496,9 @@ extern "C" int gleam_dedup_copy_noalloc(gleam_cache_t* c, const void* d_buf, siz
   d.total = total;
   d.ncalls = 1;
   d.wait_ns = c->wait_ns;
-  d.plain_copy = chk.saw_managed() ? 1u : 0u;
+  const bool packed_aligned = reinterpret_cast<uintptr_t>(one.packed) % 16 == 0;
+  d.far = chk.saw_managed() ? 1u : 0u;
+  d.plain_copy = (d.far || !aligned || !packed_aligned) ? 1u : 0u;
   set_lru(c, &d, N);
   d.skip_block = c->skip_block;  // the test hook applies to this one call, as in enqueue()
   c->skip_block = -1;
@@ -1505,10 +1507,9 @@ extern "C" int gleam_dedup_copy_noalloc(gleam_cache_t* c, const void* d_buf, siz
     grid = std::max(grid, std::min(2, c->coop_max_blocks));  // someone must be left waiting
     if (d.skip_block >= grid) d.skip_block = grid - 1;
   }
-  set_spec(c, &h, &d,
-           aligned && reinterpret_cast<uintptr_t>(one.packed) % 16 == 0 && !d.plain_copy);
-  if (small_call(c, aligned, N, n, d.skip_block)) {
-    if ((rc = cuda_err(launch_small_call(h, d, s))) != GLEAM_OK) return rc;
+  set_spec(c, &h, &d, !d.plain_copy);
+  if (small_call(c, N, n, d.skip_block)) {
+    if ((rc = cuda_err(launch_small_call(h, d, aligned, s))) != GLEAM_OK) return rc;
   } else {
     if ((rc = cuda_err(launch_hash(h, aligned, s))) != GLEAM_OK) return rc;
     if ((rc = cuda_err(launch_dedup(d, grid, pack_grid(c, N, n), s))) != GLEAM_OK) return rc;

@@ -240,7 +240,9 @@ struct DedupArgs {
   uint32_t classes;
   ClassEntry* cls_tbl;       // KEY16 classes: as many entries as tbl
   uint32_t plain_copy;       // copy misses with loads and stores, not bulk copies
-                             // (payloads or outputs in host or managed memory)
+                             // (payloads or outputs in host or managed memory, or
+                             // payloads or packed buffers not 16-byte aligned)
+  uint32_t far;              // payloads or outputs in host or managed memory
   // LRU eviction (GLEAM_EVICT_LRU; lru == 0: the other fields are unused)
   uint32_t lru;
   uint32_t epoch;            // this call's clock value
@@ -274,7 +276,7 @@ constexpr unsigned long long kHintedMaxChunk = 4096;
 cudaError_t launch_hash(const HashArgs& a, bool aligned, cudaStream_t s, bool pdl = false);
 // Whether launch_hash runs the staged XXH64 kernel for these arguments (the
 // one that can claim groups, HashArgs::claim_tbl).
-bool hash_is_staged(const HashArgs& a, bool aligned);
+bool hash_is_staged(const HashArgs& a);
 // Loads the hash kernels' device code on the current GPU (cache creation does
 // it, so that no later call loads code, which allocates device memory).
 cudaError_t load_hash_kernels();
@@ -290,11 +292,11 @@ cudaError_t launch_dedup(const DedupArgs& a, int grid, int pack_grid, cudaStream
 // `grid` blocks (see k_resolve_pack), with programmatic stream serialization.
 cudaError_t launch_resolve_pack(const DedupArgs& a, int grid, cudaStream_t s);
 // A whole call (hash, resolve and rank, pack) as one single-block kernel, for
-// calls with few chunks whose payloads suit the staged hash (16-byte aligned)
-// outside GLEAM_PAPER_IDS mode; the block hashes small_call_groups() chunks at
-// a time.
-cudaError_t launch_small_call(const HashArgs& h, const DedupArgs& a, cudaStream_t s,
-                              bool pdl = false);
+// calls with few chunks outside GLEAM_PAPER_IDS mode; the block hashes
+// small_call_groups() chunks at a time.  aligned: every payload is 16-byte
+// aligned.
+cudaError_t launch_small_call(const HashArgs& h, const DedupArgs& a, bool aligned,
+                              cudaStream_t s, bool pdl = false);
 uint32_t small_call_groups();
 cudaError_t launch_debug_insert(IndexEntry* index, uint64_t index_mask, uint32_t* slot_len,
                                 unsigned long long* slot_key, unsigned long long* dstats,

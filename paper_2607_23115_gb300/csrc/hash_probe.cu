@@ -12,10 +12,10 @@
 // hit if it is a key+length candidate and compared equal, and any other
 // candidate is compared by re-reading both copies.
 //
-// Kernels: k_hash_probe_staged (16-byte-aligned payloads: chunks stream
-// through shared memory by cp.async), k_hash_probe (any alignment: direct
-// loads), and for the paper's identifiers k_probe_paper_staged /
-// k_probe_paper (MD5 of the first 128 bytes as the key).
+// Kernels: k_hash_probe_staged (chunks stream through shared memory by
+// cp.async; a variant for payloads of any alignment), and for the paper's
+// identifiers k_probe_paper_staged / k_probe_paper (MD5 of the first 128 bytes
+// as the key; 16-byte-aligned payloads / any alignment, by direct loads).
 #include <algorithm>
 #include <cmath>
 
@@ -29,238 +29,11 @@ namespace {
 #ifndef GLEAM_HASH_THREADS
 #define GLEAM_HASH_THREADS 256
 #endif
-#ifndef GLEAM_STAGED_HASH
-#define GLEAM_STAGED_HASH 1
-#endif
 constexpr int kHashThreads = GLEAM_HASH_THREADS;
 
 
-// Lane accumulator over `ns` stripes starting at p (p already offset by 8*lane).
-template <bool kAligned>
-__device__ __forceinline__ unsigned long long lane_stripes(unsigned long long acc,
-                                                           const uint8_t* p, uint32_t ns) {
-  uint32_t s = 0;
-  if (ns >= kBatch) {
-    unsigned long long x[kBatch];
-#pragma unroll
-    for (int u = 0; u < kBatch; ++u) x[u] = load_word<kAligned>(p + (uint64_t)u * 32);
-    for (; s + 2 * kBatch <= ns; s += kBatch) {
-      unsigned long long y[kBatch];
-#pragma unroll
-      for (int u = 0; u < kBatch; ++u)
-        y[u] = load_word<kAligned>(p + (uint64_t)(s + kBatch + u) * 32);
-#pragma unroll
-      for (int u = 0; u < kBatch; ++u) acc = xstep(acc, x[u]);
-#pragma unroll
-      for (int u = 0; u < kBatch; ++u) x[u] = y[u];
-    }
-#pragma unroll
-    for (int u = 0; u < kBatch; ++u) acc = xstep(acc, x[u]);
-    s += kBatch;
-  }
-  for (; s < ns; ++s) acc = xstep(acc, load_word<kAligned>(p + (uint64_t)s * 32));
-  return acc;
-}
-
-// Lane accumulator over stripes [s0, s1) while comparing every payload word
-// with the cached copy's word at q (p, q already offset by 8*lane).  `cmp`
-// turns off, for the whole group, as soon as any word differs; diff then
-// stays non-zero.  Loads of the next batch are issued before the current one
-// is folded in.
-template <bool kAligned>
-__device__ __forceinline__ unsigned long long lane_stripes_cmp(
-    unsigned long long acc, const uint8_t* p, const uint8_t* q, uint32_t s0, uint32_t s1,
-    unsigned long long& diff, bool& cmp, unsigned gmask) {
-  constexpr int B = kBatch;
-  unsigned long long x[B], y[B];
-  uint32_t s = s0;
-  uint32_t m = min((uint32_t)B, s1 - s);
-#pragma unroll
-  for (int u = 0; u < B; ++u) {
-    x[u] = (uint32_t)u < m ? load_word<kAligned>(p + (uint64_t)(s + u) * 32) : 0ULL;
-    y[u] = (cmp && (uint32_t)u < m) ? load_arena_word(q + (uint64_t)(s + u) * 32) : x[u];
-  }
-  while (s < s1) {
-    const uint32_t sn = s + m;
-    const uint32_t mn = sn < s1 ? min((uint32_t)B, s1 - sn) : 0u;
-    unsigned long long xn[B], yn[B];
-#pragma unroll
-    for (int u = 0; u < B; ++u) {
-      xn[u] = (uint32_t)u < mn ? load_word<kAligned>(p + (uint64_t)(sn + u) * 32) : 0ULL;
-      yn[u] = (cmp && (uint32_t)u < mn) ? load_arena_word(q + (uint64_t)(sn + u) * 32) : xn[u];
-    }
-    unsigned long long d = 0;
-#pragma unroll
-    for (int u = 0; u < B; ++u) {
-      if ((uint32_t)u < m) {
-        acc = xstep(acc, x[u]);
-        d |= x[u] ^ y[u];
-      }
-    }
-    if (cmp) {
-      diff |= d;
-      unsigned long long g = diff;
-      g |= __shfl_xor_sync(gmask, g, 1);
-      g |= __shfl_xor_sync(gmask, g, 2);
-      if (g) {
-        cmp = false;
-        diff = 1;
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < B; ++u) {
-      x[u] = xn[u];
-      y[u] = yn[u];
-    }
-    s = sn;
-    m = mn;
-  }
-  return acc;
-}
-
-
-
-template <bool kAligned, bool kProbe>
-__global__ void __launch_bounds__(kHashThreads) k_hash_probe(HashArgs a) {
-  pdl_trigger();
-  pdl_wait();  // this variant reads nothing before the previous call is complete
-  const unsigned long long g = ((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) >> 2;
-  __shared__ unsigned long long s_scratch[33];
-  const uint32_t pid_b =
-      a.count > 1 ? block_find_payload(a.table, a.count,
-                                       ((unsigned long long)blockIdx.x * blockDim.x) >> 2, g,
-                                       s_scratch)
-                  : 0u;
-  if (g >= a.Ntot) return;  // whole groups leave together
-  const uint32_t lane = threadIdx.x & 3;
-  const int gbase = threadIdx.x & 28;
-  const unsigned gmask = 0xFu << gbase;
-
-  uint32_t pid = 0;
-  const uint8_t* buf;
-  unsigned long long n, base;
-  if (a.count > 1) {
-    pid = pid_b;
-    buf = a.table[pid].buf;
-    n = a.table[pid].n;
-    base = a.table[pid].chunk_base;
-  } else {
-    buf = a.one.buf;
-    n = a.one.n;
-    base = a.one.chunk_base;
-  }
-  const unsigned long long start = (g - base) * a.C;
-  const uint32_t len = (uint32_t)min(a.C, n - start);
-  const uint8_t* p = buf + start;
-  const uint32_t ns = len >> 5;
-
-  const bool speculate = kProbe && len >= kPrefixBytes;
-  const unsigned long long slots_used = kProbe ? a.dstats[ST_SLOTS_USED] : 0ULL;
-  unsigned long long hint = 0, diff = 0;
-  uint32_t hint_slot = kEmptySlot;
-  bool cmp = false;
-
-  unsigned long long h;
-  if (ns) {
-    unsigned long long acc = xlane_start(lane);
-    if (speculate) {
-      constexpr uint32_t kPre = kPrefixBytes / 32;
-      acc = lane_stripes<kAligned>(acc, p + 8 * lane, kPre);
-      const unsigned long long b0 = group_shfl(acc, gmask, gbase + 0);
-      const unsigned long long b1 = group_shfl(acc, gmask, gbase + 1);
-      const unsigned long long b2 = group_shfl(acc, gmask, gbase + 2);
-      const unsigned long long b3 = group_shfl(acc, gmask, gbase + 3);
-      hint = b0 ^ xrotl(b1, 16) ^ xrotl(b2, 32) ^ xrotl(b3, 48);
-      // an empty cache has no hints to look up
-      hint_slot = slots_used ? hint_lookup(a.hints, a.index_mask, hint, len, slots_used)
-                             : kEmptySlot;
-      const uint8_t* q = a.arena + (unsigned long long)hint_slot * a.C;
-      cmp = hint_slot != kEmptySlot;
-      if (cmp) {  // the prefix, already hashed, is compared once (payload words from L2)
-        unsigned long long d = 0;
-#pragma unroll 4
-        for (uint32_t s = 0; s < kPre; ++s) {
-          const uint64_t off = (uint64_t)s * 32 + 8 * lane;
-          d |= load_word<kAligned>(p + off) ^ load_arena_word(q + off);
-        }
-        d |= __shfl_xor_sync(gmask, d, 1);
-        d |= __shfl_xor_sync(gmask, d, 2);
-        if (d) {
-          cmp = false;
-          diff = 1;
-        }
-      }
-      acc = lane_stripes_cmp<kAligned>(acc, p + 8 * lane, q + 8 * lane, kPre, ns, diff, cmp,
-                                       gmask);
-    } else {
-      acc = lane_stripes<kAligned>(acc, p + 8 * lane, ns);
-    }
-    const unsigned long long a0 = group_shfl(acc, gmask, gbase + 0);
-    const unsigned long long a1 = group_shfl(acc, gmask, gbase + 1);
-    const unsigned long long a2 = group_shfl(acc, gmask, gbase + 2);
-    const unsigned long long a3 = group_shfl(acc, gmask, gbase + 3);
-    h = xconverge(a0, a1, a2, a3);
-  } else {
-    h = kXP5;
-  }
-  h += len;
-  h = xfinish(h, p + (uint64_t)ns * 32, len & 31);
-
-  if (a.fp_out != nullptr && lane == 0) a.fp_out[g] = h;
-  if (!kProbe) return;
-
-  // the bytes after the last full stripe, for the speculative compare
-  bool spec_equal = false;
-  if (speculate && hint_slot != kEmptySlot) {
-    unsigned long long d = diff;
-    if (cmp && lane == 0) {
-      const uint8_t* q = a.arena + (unsigned long long)hint_slot * a.C;
-      for (uint32_t k = ns * 32; k < len; ++k) d |= (unsigned long long)(p[k] ^ q[k]);
-    }
-    d |= __shfl_xor_sync(gmask, d, 1);
-    d |= __shfl_xor_sync(gmask, d, 2);
-    spec_equal = d == 0;
-  }
-
-  const unsigned long long key = a.key16 ? (h & 0xFFFFULL) : h;
-  unsigned long long pos = mix64(key) & a.index_mask;
-  bool hit = false, cand = false;
-  uint32_t hit_slot = kEmptySlot;
-  for (unsigned long long probe = 0; slots_used && probe <= a.index_mask; ++probe) {
-    const IndexEntry e = a.index[pos];
-    if (e.slot == kEmptySlot) break;
-    if (e.key == key && e.len == len) {
-      cand = true;
-      if (e.slot >= slots_used) {
-        // an entry pointing past the used slots: report, never read it
-        if (lane == 0) atomicCAS(&a.ctl->err, 0, (int)GLEAM_ERR_INTERNAL);
-      } else if (e.slot == hint_slot) {
-        if (spec_equal) {  // compared in the streaming pass
-          hit = true;
-          hit_slot = e.slot;
-          break;
-        }
-      } else if (group_equal<kAligned>(p, a.arena + (uint64_t)e.slot * a.C, len, lane, gmask)) {
-        hit = true;
-        hit_slot = e.slot;
-        break;
-      }
-    }
-    pos = (pos + 1) & a.index_mask;
-  }
-  if (lane == 0) {
-    a.ch.status[g] = hit ? kHit0 : (cand ? kMissCand : kMissNoCand);
-    a.ch.key[g] = h;  // the group key: the whole fingerprint
-    a.ch.len[g] = len;
-    a.ch.src[g] = (unsigned long long)p;
-    a.ch.pidx[g] = pid;
-    a.ch.hint[g] = hint;
-    if (hit) a.ch.ent[g] = hit_slot;
-  }
-}
-
-
-template <bool kProbe, bool kAhead, bool kVerify, bool kPrefixAsync = false, int kS = kStage>
+template <bool kProbe, bool kAhead, bool kVerify, bool kPrefixAsync = false, int kS = kStage,
+          bool kMis = false>
 __global__ void __launch_bounds__(kStagedThreads) k_hash_probe_staged(HashArgs a) {
   extern __shared__ __align__(16) uint8_t smem[];
   pdl_trigger();
@@ -268,7 +41,7 @@ __global__ void __launch_bounds__(kStagedThreads) k_hash_probe_staged(HashArgs a
   const unsigned long long nvb = (a.Ntot * 4 + kStagedThreads - 1) / kStagedThreads;
   for (unsigned long long vb = blockIdx.x; vb < nvb; vb += gridDim.x) {
     __syncthreads();  // the previous range's groups are done with the shared memory
-    staged_range<kProbe, kAhead, kVerify, kPrefixAsync, kS>(a, vb, smem);
+    staged_range<kProbe, kAhead, kVerify, kPrefixAsync, kS, kMis>(a, vb, smem);
   }
 }
 
@@ -295,11 +68,12 @@ int staged_wave_blocks() {
   return wave;
 }
 
-template <bool kProbe, bool kAhead, bool kVerify, bool kPrefixAsync = false, int kS = kStage>
+template <bool kProbe, bool kAhead, bool kVerify, bool kPrefixAsync = false, int kS = kStage,
+          bool kMis = false>
 cudaError_t launch_staged(const HashArgs& a, cudaStream_t s, bool pdl) {
   const unsigned long long threads = a.Ntot * 4;
   const unsigned sg = (unsigned)((threads + kStagedThreads - 1) / kStagedThreads);
-  if constexpr (kS == kStage && kProbe && !kPrefixAsync) {
+  if constexpr (kS == kStage && kProbe && !kPrefixAsync && !kMis) {
     // a call whose large chunks all fit one wave of the large-stage variant,
     // unless calls overlap (then the calls in flight share the SMs, and the
     // variant's larger blocks would crowd them out)
@@ -309,13 +83,14 @@ cudaError_t launch_staged(const HashArgs& a, cudaStream_t s, bool pdl) {
   }
   if constexpr (kVerify && !kPrefixAsync && kS == kStage) {
     if (a.C <= kPrefixAsyncMaxChunk)
-      return launch_staged<kProbe, kAhead, kVerify, true>(a, s, pdl);
+      return launch_staged<kProbe, kAhead, kVerify, true, kS, kMis>(a, s, pdl);
   }
-  constexpr int smem = (kStagedThreads / 4) * group_bytes(kVerify, kS);
+  constexpr int smem = (kStagedThreads / 4) * group_bytes(kVerify, kS, kMis);
   // per device and cheap: set on every launch
-  cudaFuncSetAttribute((const void*)k_hash_probe_staged<kProbe, kAhead, kVerify, kPrefixAsync, kS>,
-                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  return launch_kernel(k_hash_probe_staged<kProbe, kAhead, kVerify, kPrefixAsync, kS>, dim3(sg),
+  cudaFuncSetAttribute(
+      (const void*)k_hash_probe_staged<kProbe, kAhead, kVerify, kPrefixAsync, kS, kMis>,
+      cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  return launch_kernel(k_hash_probe_staged<kProbe, kAhead, kVerify, kPrefixAsync, kS, kMis>, dim3(sg),
                        dim3(kStagedThreads), smem, s, pdl, a);
 }
 
@@ -389,7 +164,6 @@ __device__ unsigned long long md5_prefix_key(const uint8_t* p, uint32_t m, const
   return (unsigned long long)a0 | ((unsigned long long)b0 << 32);
 }
 
-template <bool kAligned>
 __global__ void __launch_bounds__(kHashThreads) k_probe_paper(HashArgs a, Md5Table tab) {
   pdl_trigger();
   pdl_wait();
@@ -439,7 +213,7 @@ __global__ void __launch_bounds__(kHashThreads) k_probe_paper(HashArgs a, Md5Tab
         cand = true;
         if (e.slot >= slots_used) {
           if (lane == 0) atomicCAS(&a.ctl->err, 0, (int)GLEAM_ERR_INTERNAL);
-        } else if (group_equal<kAligned>(p, a.arena + (uint64_t)e.slot * a.C, len, lane, gmask)) {
+        } else if (group_equal<false>(p, a.arena + (uint64_t)e.slot * a.C, len, lane, gmask)) {
           hit = true;
           hit_slot = e.slot;
           break;
@@ -633,51 +407,36 @@ cudaError_t load_hash_kernels() {
   return cudaFuncGetAttributes(&fa, k_hash_probe_staged<true, false, true>);
 }
 
-bool hash_is_staged(const HashArgs& a, bool aligned) {
-#if GLEAM_STAGED_HASH
-  return a.Ntot > 0 && !(a.index != nullptr && a.paper) && aligned && (a.C % 32 == 0 || a.Ntot == 1);
-#else
-  return false;
-#endif
-}
+bool hash_is_staged(const HashArgs& a) { return a.Ntot > 0 && !(a.index != nullptr && a.paper); }
 
 cudaError_t launch_hash(const HashArgs& a, bool aligned, cudaStream_t s, bool pdl) {
   if (a.Ntot == 0) return cudaSuccess;
-  const unsigned long long threads = a.Ntot * 4;
-  const unsigned grid = (unsigned)((threads + kHashThreads - 1) / kHashThreads);
   const bool probe = a.index != nullptr;
   if (probe && a.paper) {
     static const Md5Table tab = md5_table();
-#if GLEAM_STAGED_HASH
-    if (aligned && a.C % 32 == 0) {
+    const unsigned long long threads = a.Ntot * 4;
+    if (aligned) {
       const unsigned sg = (unsigned)((threads + kStagedThreads - 1) / kStagedThreads);
       return launch_kernel(k_probe_paper_staged, dim3(sg), dim3(kStagedThreads), kStagedSmem, s,
                            pdl, a, tab);
     }
-#endif
-    return aligned ? launch_kernel(k_probe_paper<true>, dim3(grid), dim3(kHashThreads), 0, s,
-                                   pdl, a, tab)
-                   : launch_kernel(k_probe_paper<false>, dim3(grid), dim3(kHashThreads), 0, s,
-                                   pdl, a, tab);
+    const unsigned grid = (unsigned)((threads + kHashThreads - 1) / kHashThreads);
+    return launch_kernel(k_probe_paper, dim3(grid), dim3(kHashThreads), 0, s, pdl, a, tab);
   }
-#if GLEAM_STAGED_HASH
-  if (aligned && (a.C % 32 == 0 || a.Ntot == 1)) {
-    // no cached copy is streamed when only fingerprints are wanted or the
-    // cache holds no chunk (or too few to be worth the hint lookups): the
-    // variant without those buffers
-    if (!probe) return launch_staged<false, false, false>(a, s, pdl);
-    if (a.no_hints)
-      return a.spec_mode ? launch_staged<true, true, false>(a, s, pdl)
-                         : launch_staged<true, false, false>(a, s, pdl);
-    return a.spec_mode ? launch_staged<true, true, true>(a, s, pdl)
-                       : launch_staged<true, false, true>(a, s, pdl);
+  // no cached copy is streamed when only fingerprints are wanted or the cache
+  // holds no chunk (or too few to be worth the hint lookups): the variant
+  // without those buffers
+  if (!aligned) {  // no write-through: its 16-byte stores want aligned payloads
+    if (!probe) return launch_staged<false, false, false, false, kStage, true>(a, s, pdl);
+    if (a.no_hints) return launch_staged<true, false, false, false, kStage, true>(a, s, pdl);
+    return launch_staged<true, false, true, false, kStage, true>(a, s, pdl);
   }
-#endif
-  const dim3 g3(grid), b3(kHashThreads);
-  if (aligned && probe) return launch_kernel(k_hash_probe<true, true>, g3, b3, 0, s, pdl, a);
-  if (aligned) return launch_kernel(k_hash_probe<true, false>, g3, b3, 0, s, pdl, a);
-  if (probe) return launch_kernel(k_hash_probe<false, true>, g3, b3, 0, s, pdl, a);
-  return launch_kernel(k_hash_probe<false, false>, g3, b3, 0, s, pdl, a);
+  if (!probe) return launch_staged<false, false, false>(a, s, pdl);
+  if (a.no_hints)
+    return a.spec_mode ? launch_staged<true, true, false>(a, s, pdl)
+                       : launch_staged<true, false, false>(a, s, pdl);
+  return a.spec_mode ? launch_staged<true, true, true>(a, s, pdl)
+                     : launch_staged<true, false, true>(a, s, pdl);
 }
 
 }  // namespace gleam

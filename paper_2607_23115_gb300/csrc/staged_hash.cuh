@@ -89,15 +89,20 @@ __device__ __forceinline__ bool group_equal(const uint8_t* p, const uint8_t* q, 
 // strided across the lanes, kBatch of them per lane in flight, leaving early
 // once any word differs.  Eight groups' worth of lanes take a 64 KiB compare
 // in 32 rounds of loads where one group's four lanes take 256.
+// kMis: p may have any alignment.
+template <bool kMis>
 __device__ __forceinline__ bool lanes_equal(const uint8_t* p, const uint8_t* q, uint32_t len,
                                             unsigned wmask, uint32_t wl, uint32_t nl) {
   const uint32_t nw = len >> 3;
+  const bool words = !kMis || ((uintptr_t)p & 7) == 0;
   for (uint32_t w0 = 0; w0 < nw; w0 += kBatch * nl) {
     unsigned long long diff = 0;
 #pragma unroll
     for (int u = 0; u < kBatch; ++u) {
       const uint32_t w = w0 + u * nl + wl;
-      if (w < nw) diff |= load_word<true>(p + 8ull * w) ^ load_arena_word(q + 8ull * w);
+      if (w < nw)
+        diff |= (words ? load_word<true>(p + 8ull * w) : load_word<false>(p + 8ull * w)) ^
+                load_arena_word(q + 8ull * w);
     }
     if (__any_sync(wmask, diff != 0)) return false;
   }
@@ -116,7 +121,7 @@ __device__ __forceinline__ unsigned present_lanes(unsigned long long vb, unsigne
 }
 
 // ---------------------------------------------------------------------------
-// Staged variant for 16-byte-aligned payloads.  Each 4-thread group streams
+// The staged routine.  Each 4-thread group streams
 // its chunk through shared memory in kStage-byte stages with asynchronous
 // 16-byte global->shared copies (kDepth stages in flight, no registers held),
 // and the cached copy named by the prefix hint streams alongside into a
@@ -146,8 +151,13 @@ constexpr int kDepth = GLEAM_STAGE_DEPTH;                   // stages in flight
 // A group's stage buffers: kDepth stages of its chunk and, when it may
 // compare against a cached copy (verify), kDepth stages of that copy too
 // (+32: bank skew).
-__host__ __device__ constexpr int group_bytes(bool verify, int stage = kStage) {
-  return kDepth * (verify ? 2 : 1) * stage + 32;
+// mis: payload stages of any alignment, read as the 16-byte pieces they lie in
+// (one more per stage); groups are still 32 bytes off a multiple of the 128
+// bytes of all banks, so that four groups' words meet no bank twice.
+__host__ __device__ constexpr int group_bytes(bool verify, int stage = kStage, bool mis = false) {
+  return mis ? kDepth * ((verify ? 2 : 1) * stage + 16) +
+                   ((32 - kDepth * ((verify ? 2 : 1) * stage + 16)) & 127)
+             : kDepth * (verify ? 2 : 1) * stage + 32;
 }
 // Stage size of the variant for calls that leave most of the GPU idle (fewer
 // chunks than one wave of it holds, chunks of at least kBigStageMinChunk):
@@ -160,10 +170,18 @@ constexpr int kGroupBytes = group_bytes(true);
 constexpr int kStagedThreads = GLEAM_STAGED_THREADS;
 constexpr int kStagedSmem = (kStagedThreads / 4) * kGroupBytes;
 static_assert(kStage == (int)kPrefixBytes, "stage 0 must be the hinted prefix");
+static_assert(group_bytes(true, kStage, true) == kGroupBytes || kDepth != 2,
+              "payloads of any alignment fit the same two-stage region");
 static_assert(kStagedSmem >= 33 * 8, "the payload search borrows 33 words of the stage buffers");
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
   asm volatile("cp.async.cg.shared.global.L2::256B [%0], [%1], 16;" ::"r"(dst), "l"(src)
+               : "memory");
+}
+// The first `bytes` (1..16) of a 16-byte piece, the rest filled with zeros.
+__device__ __forceinline__ void cp_async16_upto(uint32_t dst, const void* src, uint32_t bytes) {
+  asm volatile("cp.async.cg.shared.global.L2::256B [%0], [%1], 16, %2;" ::"r"(dst), "l"(src),
+               "r"(bytes)
                : "memory");
 }
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
@@ -195,6 +213,28 @@ __device__ __forceinline__ void stage_copy(uint32_t dst, const uint8_t* src, uin
   }
 }
 
+// stage_copy for a payload of any alignment.  src: the stage's first byte
+// rounded down to 16; win: bytes from there to the stage's last byte (at most
+// kS + 15).  The pieces that reach past the payload [lo, hi) are read up to its
+// ends only.
+template <int kS>
+__device__ __forceinline__ void stage_copy_any(uint32_t dst, uint8_t* dstp, const uint8_t* src,
+                                               uint32_t win, uint32_t lane, const uint8_t* lo,
+                                               const uint8_t* hi) {
+  const uint32_t lim = (uint32_t)min((unsigned long long)(hi - src), (unsigned long long)kS + 16);
+  const uint32_t o0 = src < lo ? 16u : 0u;  // the payload's first piece, if it starts inside one
+  if (o0 && lane == 0)
+    for (uint32_t b = (uint32_t)(lo - src); b < 16 && b < win; ++b) dstp[b] = src[b];
+  auto piece = [&](uint32_t off) {
+    if (off < o0 || off >= win) return;
+    if (off + 16 <= lim) cp_async16(dst + off, src + off);
+    else cp_async16_upto(dst + off, src + off, lim - off);
+  };
+#pragma unroll
+  for (int j = 0; j < kS / 64; ++j) piece((uint32_t)j * 64 + lane * 16);
+  if (lane == 0) piece((uint32_t)kS);
+}
+
 // The chunks of block-sized range vb (blockDim.x / 4 consecutive chunks); the
 // shared memory holds one region of group_bytes(kVerify) per group.  kAhead:
 // with the write-through of likely misses (written ahead of the pack step).
@@ -202,11 +242,20 @@ __device__ __forceinline__ void stage_copy(uint32_t dst, const uint8_t* src, uin
 // (for a cache that holds no chunk, or too few to be worth the lookups), so
 // twice as many groups fit an SM; a key+length candidate, if any, is still
 // compared with direct loads.
+//
+// kMis: payloads (and fingerprinted chunks) of any alignment.  Each chunk is
+// read in the 16-byte pieces it lies in, and a lane's word is put together from
+// the one or two aligned 8-byte words of shared memory that hold it.  Its
+// stages are 16 bytes longer, and the extra load and shifts are why aligned
+// payloads keep the other variant.  Loading such payloads byte by byte instead,
+// as before, the hash of 260 MB at 8-byte alignment took 388 us, and the whole
+// call 1,489 us against 245 us now (16 KiB chunks, a tenth of them changed).
 template <bool kProbe, bool kAhead = false, bool kVerify = true, bool kPrefixAsync = false,
-          int kS = kStage>
+          int kS = kStage, bool kMis = false>
 __device__ __forceinline__ void staged_range(const HashArgs& a, unsigned long long vb,
                                              uint8_t* smem) {
   static_assert(kS % kPrefixBytes == 0 && kS % 256 == 0, "stages hold whole prefixes and batches");
+  static_assert(!(kMis && kAhead), "chunks are written ahead in aligned 16-byte pieces");
   const unsigned long long g = (vb * blockDim.x + threadIdx.x) >> 2;
   // the payload search borrows the start of the stage buffers (no static
   // shared memory: any would cost this kernel a fifth of its bandwidth)
@@ -218,10 +267,12 @@ __device__ __forceinline__ void staged_range(const HashArgs& a, unsigned long lo
   const uint32_t lane = threadIdx.x & 3;
   const int gbase = threadIdx.x & 28;
   const unsigned gmask = 0xFu << gbase;
-  uint8_t* region = smem + (threadIdx.x >> 2) * group_bytes(kVerify, kS);
+  uint8_t* region = smem + (threadIdx.x >> 2) * group_bytes(kVerify, kS, kMis);
   const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(region);
-  // stage buffer t % kDepth: payload at [0, kS), cached copy at [kS, 2 kS)
-  constexpr uint32_t kBuf = (kVerify ? 2 : 1) * kS;  // one stage's buffers
+  // stage buffer t % kDepth: payload at [0, kS) (kMis: 16 bytes more), cached
+  // copy at [kPay, kPay + kS)
+  constexpr uint32_t kPay = kS + (kMis ? 16 : 0);
+  constexpr uint32_t kBuf = kPay + (kVerify ? kS : 0);  // one stage's buffers
   auto pay_s = [&](uint32_t t) { return sbase + (t % kDepth) * kBuf; };
   auto pay_p = [&](uint32_t t) { return region + (t % kDepth) * kBuf; };
 
@@ -245,6 +296,14 @@ __device__ __forceinline__ void staged_range(const HashArgs& a, unsigned long lo
   const uint32_t full = ns * 32;                       // bytes in whole stripes
   const uint32_t nst = (full + kS - 1) / kS;   // stages
   auto sbytes = [&](uint32_t t) { return min((uint32_t)kS, full - t * kS); };
+  const uint32_t mis = kMis ? (uint32_t)((uintptr_t)p & 15) : 0u;
+  auto pay_copy = [&](uint32_t t) {  // this lane's share of payload stage t
+    if constexpr (kMis)
+      stage_copy_any<kS>(pay_s(t), pay_p(t), p - mis + (unsigned long long)t * kS, mis + sbytes(t),
+                         lane, buf, buf + n);
+    else
+      stage_copy<kS>(pay_s(t), p + (unsigned long long)t * kS, sbytes(t), lane);
+  };
 
   const bool speculate = kProbe && len >= kPrefixBytes;
   // slots in use as the hint lookups see them; with a late wait (calls that
@@ -270,15 +329,15 @@ __device__ __forceinline__ void staged_range(const HashArgs& a, unsigned long lo
   // prologue: payload stages 0 .. kDepth-2
 #pragma unroll
   for (int t = 0; t < kDepth - 1; ++t) {
-    if ((uint32_t)t < nst) stage_copy<kS>(pay_s(t), p + t * kS, sbytes(t), lane);
+    if ((uint32_t)t < nst) pay_copy((uint32_t)t);
     cp_commit();
   }
   for (uint32_t t = 0; t < nst; ++t) {
     // issue stage t + kDepth - 1 into the buffer consumed at t - 1
     const uint32_t tn = t + kDepth - 1;
     if (tn < nst) {
-      stage_copy<kS>(pay_s(tn), p + (unsigned long long)tn * kS, sbytes(tn), lane);
-      if (cmp) stage_copy<kS>(pay_s(tn) + kS, q + (unsigned long long)tn * kS, sbytes(tn), lane);
+      pay_copy(tn);
+      if (cmp) stage_copy<kS>(pay_s(tn) + kPay, q + (unsigned long long)tn * kS, sbytes(tn), lane);
     }
     cp_commit();
     // groups committed so far, oldest first: prologue stages, then one per
@@ -294,6 +353,19 @@ __device__ __forceinline__ void staged_range(const HashArgs& a, unsigned long lo
     auto word = [&](const uint8_t* b, uint32_t s) {
       return *reinterpret_cast<const unsigned long long*>(b + s * 32 + lane * 8);
     };
+    auto pword = [&](uint32_t s) {  // the lane's payload word of stripe s
+      if constexpr (kMis) {
+        const uint8_t* b = sp + (mis & 8) + s * 32 + lane * 8;
+        unsigned long long v = *reinterpret_cast<const unsigned long long*>(b);
+        if (mis & 7) {
+          const uint32_t sh = (mis & 7) * 8;
+          v = (v >> sh) | (*reinterpret_cast<const unsigned long long*>(b + 8) << (64 - sh));
+        }
+        return v;
+      } else {
+        return word(sp, s);
+      }
+    };
     if (sst == (uint32_t)kS / 32) {
       // a whole stage, eight stripes at a time: the loads and the compare
       // overlap the XXH64 chain instead of waiting in it
@@ -301,28 +373,28 @@ __device__ __forceinline__ void staged_range(const HashArgs& a, unsigned long lo
       for (uint32_t h = 0; h < (uint32_t)kS / 32; h += 8) {
         unsigned long long w[8];
 #pragma unroll
-        for (uint32_t u = 0; u < 8; ++u) w[u] = word(sp, h + u);
+        for (uint32_t u = 0; u < 8; ++u) w[u] = pword(h + u);
         if (cmp && t > 0) {
 #pragma unroll
-          for (uint32_t u = 0; u < 8; ++u) d |= w[u] ^ word(sp + kS, h + u);
+          for (uint32_t u = 0; u < 8; ++u) d |= w[u] ^ word(sp + kPay, h + u);
         }
 #pragma unroll
         for (uint32_t u = 0; u < 8; ++u) acc = xstep(acc, w[u]);
         if (kS > (int)kPrefixBytes && h + 8 == kPrefixBytes / 32) acc_pre = acc;
       }
     } else if (cmp && t > 0) {
-      const uint8_t* sq = sp + kS;
+      const uint8_t* sq = sp + kPay;
 #pragma unroll 4
       for (uint32_t s = 0; s < sst; ++s) {
-        const unsigned long long w = *reinterpret_cast<const unsigned long long*>(sp + s * 32 + lane * 8);
-        const unsigned long long c = *reinterpret_cast<const unsigned long long*>(sq + s * 32 + lane * 8);
+        const unsigned long long w = pword(s);
+        const unsigned long long c = word(sq, s);
         acc = xstep(acc, w);
         d |= w ^ c;
       }
     } else {
 #pragma unroll 4
       for (uint32_t s = 0; s < sst; ++s) {
-        acc = xstep(acc, *reinterpret_cast<const unsigned long long*>(sp + s * 32 + lane * 8));
+        acc = xstep(acc, pword(s));
         if (kS > (int)kPrefixBytes && s + 1 == kPrefixBytes / 32) acc_pre = acc;
       }
     }
@@ -350,19 +422,18 @@ __device__ __forceinline__ void staged_range(const HashArgs& a, unsigned long lo
           // the cached copy's prefix into the free half of stage buffer 0, in
           // a group of its own, and its next stages behind it: one round trip
           // for both
-          stage_copy<kS>(pay_s(0) + kS, q, kS == (int)kPrefixBytes ? (uint32_t)kS : sbytes(0), lane);
+          stage_copy<kS>(pay_s(0) + kPay, q, kS == (int)kPrefixBytes ? (uint32_t)kS : sbytes(0), lane);
           cp_commit();
         } else {
           // stage 0 (the prefix, and more in a larger stage), still in its
           // buffer, against the cached copy's
 #pragma unroll 4
           for (uint32_t s = 0; s < (kS == (int)kPrefixBytes ? (uint32_t)kS / 32 : sst); ++s)
-            d |= *reinterpret_cast<const unsigned long long*>(sp + s * 32 + lane * 8) ^
-                 load_arena_word(q + s * 32 + lane * 8);
+            d |= pword(s) ^ load_arena_word(q + s * 32 + lane * 8);
         }
         // the cached copy of the stages already in flight
         for (uint32_t tt = 1; tt < (uint32_t)kDepth && tt < nst; ++tt)
-          stage_copy<kS>(pay_s(tt) + kS, q + (unsigned long long)tt * kS, sbytes(tt), lane);
+          stage_copy<kS>(pay_s(tt) + kPay, q + (unsigned long long)tt * kS, sbytes(tt), lane);
       }
     }
     if (t == 0) cp_commit();  // the late group (empty without a hint)
@@ -372,10 +443,10 @@ __device__ __forceinline__ void staged_range(const HashArgs& a, unsigned long lo
       __syncwarp(gmask);
       if constexpr (kS == (int)kPrefixBytes) {
 #pragma unroll
-        for (uint32_t s = 0; s < (uint32_t)kS / 32; ++s) d |= word(sp, s) ^ word(sp + kS, s);
+        for (uint32_t s = 0; s < (uint32_t)kS / 32; ++s) d |= pword(s) ^ word(sp + kPay, s);
       } else {
 #pragma unroll 4
-        for (uint32_t s = 0; s < sst; ++s) d |= word(sp, s) ^ word(sp + kS, s);
+        for (uint32_t s = 0; s < sst; ++s) d |= pword(s) ^ word(sp + kPay, s);
       }
     }
     if (cmp) {
@@ -496,7 +567,7 @@ __device__ __forceinline__ void staged_range(const HashArgs& a, unsigned long lo
             __shfl_sync(wmask, reinterpret_cast<unsigned long long>(p), src));
         const uint32_t slot = __shfl_sync(wmask, want, src);
         const uint32_t ls = __shfl_sync(wmask, len, src);
-        const bool eq = lanes_equal(ps, a.arena + (uint64_t)slot * a.C, ls, wmask, wl, nl);
+        const bool eq = lanes_equal<kMis>(ps, a.arena + (uint64_t)slot * a.C, ls, wmask, wl, nl);
         if (gbase == src && eq) {
           hit = true;
           hit_slot = slot;
