@@ -15,6 +15,9 @@
 
 using namespace gleam;
 
+// Limit of every device-side wait unless GLEAM_DEBUG_WAIT_LIMIT_NS changes it.
+constexpr unsigned long long kDefaultWaitNs = 4000000000ULL;
+
 struct gleam_cache {
   int device = 0;
   size_t capacity_bytes = 0;
@@ -77,7 +80,7 @@ struct gleam_cache {
   uint32_t* spec_mirror = nullptr;  // page-locked, mapped: [0] as of the last finished call
   int spec_hook = 0;                // GLEAM_DEBUG_SPECULATE: 0 auto, 1 always, 2 never
 
-  unsigned long long wait_ns = 4000000000ULL;
+  unsigned long long wait_ns = kDefaultWaitNs;
   int skip_block = -1;
 
   // id (cudaStreamGetId) of the stream `done` was last recorded on: a call on
@@ -675,6 +678,7 @@ int enqueue(gleam_cache* c, const gleam_payload_t* payloads, uint64_t count,
   h.paper = (c->flags & GLEAM_PAPER_IDS) ? 1u : 0u;
   h.ch = c->ch;
   h.ctl = c->ctl;
+  h.wait_ns = c->wait_ns;
   // slots_bound: an upper bound of the used slots
   h.no_hints = c->slots_bound == 0 ||
                        (c->C <= kHintedMaxChunk && c->slots_bound * kHintedMinRatio < Ntot)
@@ -701,6 +705,7 @@ int enqueue(gleam_cache* c, const gleam_payload_t* payloads, uint64_t count,
   d.classes = d.key16 && !d.paper ? 1u : 0u;
   d.cls_tbl = c->cls_tbl;
   d.far = (host_payloads || chk.saw_managed()) ? 1u : 0u;
+  h.far = d.far;
   d.plain_copy = (d.far || !aligned || !packed_aligned) ? 1u : 0u;
   d.tbl = c->tbl;
   d.tbl_mask = tcap - 1;
@@ -978,6 +983,8 @@ int gleam_fingerprint(const void* d_buf, size_t n, size_t chunk_bytes, uint64_t*
   h.Ntot = N;
   h.C = C;
   h.fp_out = reinterpret_cast<unsigned long long*>(d_out);
+  h.wait_ns = kDefaultWaitNs;
+  h.far = chk.saw_managed() ? 1u : 0u;
   const bool aligned = (reinterpret_cast<uintptr_t>(d_buf) % 16 == 0) && (N == 1 || C % 16 == 0);
   return cuda_err(launch_hash(h, aligned, reinterpret_cast<cudaStream_t>(stream)));
 }
@@ -1466,6 +1473,7 @@ extern "C" int gleam_dedup_copy_noalloc(gleam_cache_t* c, const void* d_buf, siz
   h.paper = (c->flags & GLEAM_PAPER_IDS) ? 1u : 0u;
   h.ch = ch;
   h.ctl = ctl;
+  h.wait_ns = c->wait_ns;
   h.no_hints = c->slots_bound == 0 ||
                        (c->C <= kHintedMaxChunk && c->slots_bound * kHintedMinRatio < N)
                    ? 1u : 0u;
@@ -1498,6 +1506,7 @@ extern "C" int gleam_dedup_copy_noalloc(gleam_cache_t* c, const void* d_buf, siz
   d.wait_ns = c->wait_ns;
   const bool packed_aligned = reinterpret_cast<uintptr_t>(one.packed) % 16 == 0;
   d.far = chk.saw_managed() ? 1u : 0u;
+  h.far = d.far;
   d.plain_copy = (d.far || !aligned || !packed_aligned) ? 1u : 0u;
   set_lru(c, &d, N);
   d.skip_block = c->skip_block;  // the test hook applies to this one call, as in enqueue()

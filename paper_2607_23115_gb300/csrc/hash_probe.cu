@@ -22,6 +22,7 @@
 #include "gleam_internal.cuh"
 #include "xxh64_device.cuh"
 #include "staged_hash.cuh"
+#include "lone_hash.cuh"
 
 namespace gleam {
 namespace {
@@ -391,6 +392,70 @@ __global__ void __launch_bounds__(kStagedThreads) k_probe_paper_staged(HashArgs 
   }
 }
 
+// SMs of the GPU (the machine's GPUs are all alike); 0 if unknown.
+int sm_count() {
+  static int n = -1;
+  if (n < 0) {
+    int dev = 0, v = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+      cudaGetLastError();
+      return 0;
+    }
+    n = v;
+  }
+  return n;
+}
+
+// Whether a call hashes with a warp per chunk (k_hash_lone) instead of the
+// staged kernel: its chunks fit one wave of it (16 to an SM), so that each is
+// a chain that the call waits for.  Per call, back to back, all chunks cached,
+// warp per chunk against staged: 64 KiB chunks, 100 / 1,200 / 2,400 of them, 49
+// / 60 / 73 us against 84 / 99 / 103; 16 KiB chunks 23 / 28 / 34 against 37 /
+// 41 / 45; 4 KiB chunks 12 / 19 / 19 against 16 / 20 / 21; 1 KiB chunks, whose
+// 32 rounds are over when the others' second stage arrives, 11.5 / 17.5 / 18.4
+// against 11.8 / 16.9 / 16.5.  With more chunks than that the DRAM is the bound
+// and the staged kernel streams better (6,658 chunks of 64 KiB: 311 us the
+// call, 345 with this one).  Calls that overlap hide each other's chains: only
+// large chunks, and few of them, gain there (64 KiB, 100 / 600 chunks: 12 / 20
+// us against 25 / 27, but 1,200 chunks 35 against 30).  Payloads in host memory
+// stay with the staged kernel, whose 64-byte reads of eight chunks at a time
+// cross the CPU-GPU link faster than a chunk's 512 bytes (451 chunks of 64
+// KiB: 227 us the call, 314 with this one).
+constexpr unsigned long long kLoneMinChunk = 4096, kLoneMinChunkOverlap = 32768;
+
+bool lone_call(const HashArgs& a) {
+  const unsigned long long sms = sm_count();
+  return !a.far && (a.wait_late ? a.C >= kLoneMinChunkOverlap && a.Ntot <= 4 * sms
+                                : a.C >= kLoneMinChunk && a.Ntot <= 2 * kLoneChunks * sms);
+}
+
+template <bool kProbe, uint32_t kD>
+cudaError_t launch_lone(const HashArgs& a, uint32_t per, cudaStream_t s, bool pdl) {
+  const uint32_t smem = per * lone_bytes(kD);
+  cudaFuncSetAttribute((const void*)k_hash_lone<kProbe, kD>,
+                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  return launch_kernel(k_hash_lone<kProbe, kD>, dim3((unsigned)((a.Ntot + per - 1) / per)),
+                       dim3(32 * (1 + per)), smem, s, pdl, a, per);
+}
+
+template <bool kProbe>
+cudaError_t launch_lone(const HashArgs& a, cudaStream_t s, bool pdl) {
+  // as few chunks to a block as keep every block resident at once; the fewer,
+  // the more stages in flight
+  const unsigned long long room = 2ull * sm_count();
+  const uint32_t per =
+      (uint32_t)std::min<unsigned long long>(kLoneChunks, (a.Ntot + room - 1) / room);
+  static_assert(2 * (kLoneChunks * lone_bytes(4) + 3072) <= 228 * 1024 &&
+                    6 * lone_bytes(6) <= kLoneChunks * lone_bytes(4) &&
+                    4 * lone_bytes(8) <= kLoneChunks * lone_bytes(4),
+                "two blocks per SM");
+  if (a.wait_late) return launch_lone<kProbe, 4>(a, per, s, pdl);  // calls share the SMs
+  if (per <= 4) return launch_lone<kProbe, 8>(a, per, s, pdl);
+  if (per <= 6) return launch_lone<kProbe, 6>(a, per, s, pdl);
+  return launch_lone<kProbe, 4>(a, per, s, pdl);
+}
+
 Md5Table md5_table() {
   Md5Table t;
   for (int i = 0; i < 64; ++i)
@@ -423,6 +488,7 @@ cudaError_t launch_hash(const HashArgs& a, bool aligned, cudaStream_t s, bool pd
     const unsigned grid = (unsigned)((threads + kHashThreads - 1) / kHashThreads);
     return launch_kernel(k_probe_paper, dim3(grid), dim3(kHashThreads), 0, s, pdl, a, tab);
   }
+  if (lone_call(a)) return probe ? launch_lone<true>(a, s, pdl) : launch_lone<false>(a, s, pdl);
   // no cached copy is streamed when only fingerprints are wanted or the cache
   // holds no chunk (or too few to be worth the hint lookups): the variant
   // without those buffers

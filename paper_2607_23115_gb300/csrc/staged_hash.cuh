@@ -235,6 +235,178 @@ __device__ __forceinline__ void stage_copy_any(uint32_t dst, uint8_t* dstp, cons
   if (lane == 0) piece((uint32_t)kS);
 }
 
+// What is known of a chunk once its whole stripes have been hashed: the lane's
+// accumulator, and the outcome of the speculative verify (hint_slot, or
+// kEmptySlot; diff: a difference the lane saw; cmp: it saw none).
+struct ChunkEnd {
+  unsigned long long g;
+  const uint8_t* p;
+  uint32_t len, lane, pid, hint_slot;
+  int gbase;
+  unsigned long long acc, hint, hint_key, diff, slots_used;
+  bool cmp, ahead;
+};
+
+// Finishes a chunk: fingerprint, index probe, verify of the candidates that
+// the streaming pass did not compare, the chunk's record and its group claim.
+// Called by the four lanes of each chunk; wmask: the warp's lanes that hold one
+// (a prefix of the warp, all of which call this).
+template <bool kProbe, bool kAhead, bool kMis>
+__device__ __forceinline__ void record_chunk(const HashArgs& a, const ChunkEnd& c,
+                                             unsigned wmask) {
+  const unsigned long long g = c.g, slots_used = c.slots_used, hint = c.hint;
+  const unsigned long long acc = c.acc, hint_key = c.hint_key, diff = c.diff;
+  const uint8_t* p = c.p;
+  const uint32_t len = c.len, lane = c.lane, pid = c.pid, hint_slot = c.hint_slot;
+  const int gbase = c.gbase;
+  const unsigned gmask = 0xFu << gbase;
+  const bool cmp = c.cmp, ahead = c.ahead;
+  const uint32_t ns = len >> 5, full = ns * 32;
+  const bool speculate = kProbe && len >= kPrefixBytes;
+  unsigned long long h;
+  if (ns) {
+    const unsigned long long a0 = group_shfl(acc, gmask, gbase + 0);
+    const unsigned long long a1 = group_shfl(acc, gmask, gbase + 1);
+    const unsigned long long a2 = group_shfl(acc, gmask, gbase + 2);
+    const unsigned long long a3 = group_shfl(acc, gmask, gbase + 3);
+    h = xconverge(a0, a1, a2, a3);
+  } else {
+    h = kXP5;
+  }
+  h += len;
+  h = xfinish(h, p + full, len & 31);
+
+  if (a.fp_out != nullptr && lane == 0) a.fp_out[g] = h;
+  if (!kProbe) return;
+  // with a late wait, the cache's previous calls are complete from here on:
+  // the probe sees their inserts (candidates at or above slots_used are
+  // compared like any other), and every write of this kernel follows
+  unsigned long long slots_now = slots_used;
+  if (a.wait_late) {
+    pdl_wait();
+    slots_now = *reinterpret_cast<const volatile unsigned long long*>(&a.dstats[ST_SLOTS_USED]);
+  }
+
+  bool spec_equal = false;
+  if (speculate && hint_slot != kEmptySlot) {
+    unsigned long long dd = diff;
+    if (cmp && lane == 0) {
+      const uint8_t* q = a.arena + (unsigned long long)hint_slot * a.C;
+      for (uint32_t k = full; k < len; ++k) dd |= (unsigned long long)(p[k] ^ q[k]);
+    }
+    dd |= __shfl_xor_sync(gmask, dd, 1);
+    dd |= __shfl_xor_sync(gmask, dd, 2);
+    spec_equal = dd == 0;
+  }
+
+  const unsigned long long key = a.key16 ? (h & 0xFFFFULL) : h;
+  bool hit = false, cand = false;
+  uint32_t hit_slot = kEmptySlot;
+  if (slots_now) {
+    // The linear probe, in order.  A key+length candidate other than the
+    // verified hint is compared by the whole warp: each group walks its probe
+    // up to its next such candidate, then the warp compares the pending ones,
+    // one group's at a time, and the groups whose candidate differs walk on.
+    const uint32_t wl = threadIdx.x & 31, nl = __popc(wmask);
+    unsigned long long pos = mix64(key) & a.index_mask, probe = 0;
+    // the hinted slot holds these very bytes and this fingerprint: the index
+    // lists it under this key and length (both are written for every stored
+    // chunk), so it is the hit and the probe can be skipped
+    bool done = false;
+    if (spec_equal && hint_key == h) {
+      hit = true;
+      hit_slot = hint_slot;
+      done = true;
+    }
+    for (;;) {
+      uint32_t want = kEmptySlot;  // a candidate for the warp to compare
+      while (!done) {
+        if (probe > a.index_mask) {
+          done = true;
+          break;
+        }
+        const IndexEntry e = a.index[pos];
+        if (e.slot == kEmptySlot) {
+          done = true;
+          break;
+        }
+        pos = (pos + 1) & a.index_mask;
+        ++probe;
+        if (e.key == key && e.len == len) {
+          cand = true;
+          if (e.slot >= slots_now) {
+            if (lane == 0) atomicCAS(&a.ctl->err, 0, (int)GLEAM_ERR_INTERNAL);
+          } else if (e.slot == hint_slot) {
+            if (spec_equal) {
+              hit = true;
+              hit_slot = e.slot;
+              done = true;
+            }
+          } else {
+            want = e.slot;
+            break;
+          }
+        }
+      }
+      const unsigned pend = __ballot_sync(wmask, want != kEmptySlot) & 0x11111111u;
+      if (!pend) break;
+      for (unsigned m = pend; m; m &= m - 1) {
+        const int src = __ffs(m) - 1;
+        const uint8_t* ps = reinterpret_cast<const uint8_t*>(
+            __shfl_sync(wmask, reinterpret_cast<unsigned long long>(p), src));
+        const uint32_t slot = __shfl_sync(wmask, want, src);
+        const uint32_t ls = __shfl_sync(wmask, len, src);
+        const bool eq = lanes_equal<kMis>(ps, a.arena + (uint64_t)slot * a.C, ls, wmask, wl, nl);
+        if (gbase == src && eq) {
+          hit = true;
+          hit_slot = slot;
+          done = true;
+        }
+      }
+    }
+  }
+  if (lane == 0) {
+    a.ch.status[g] = hit ? kHit0 : (cand ? kMissCand : kMissNoCand);
+    a.ch.key[g] = h;  // the group key: the whole fingerprint
+    a.ch.len[g] = len;
+    a.ch.src[g] = (unsigned long long)p;
+    a.ch.pidx[g] = pid;
+    a.ch.hint[g] = hint;
+    if (kAhead) a.ch.spec[g] = ahead ? 1 : 0;
+    if (hit) {
+      a.ch.ent[g] = hit_slot;
+    } else if (kProbe && a.claim_tbl != nullptr) {
+      // the miss's (group key, length) entry of the per-call table, claimed
+      // with one 64-bit CAS that also stores a 32-bit tag of the pair (where
+      // the resolve kernel keeps a minimum): an entry found holding the same
+      // tag may be the chunk's group, which sends the call down the general
+      // path (shared_groups), where the groups are claimed again by the whole
+      // key; a different tag is another group's entry
+      const unsigned long long mixed = mix64(h ^ ((unsigned long long)len << 40));
+      const unsigned long long tag = mixed >> 32;
+      unsigned long long pos = mixed & a.claim_mask;
+      uint32_t e = 0xFFFFFFFFu;
+      for (unsigned long long probe = 0; probe <= a.claim_mask; ++probe) {
+        const unsigned long long old =
+            atomicCAS(reinterpret_cast<unsigned long long*>(&a.claim_tbl[pos]), 0ull,
+                      (tag << 32) | ((unsigned long long)g + 1ull));
+        if (old == 0) {
+          e = (uint32_t)pos;
+          break;
+        }
+        if ((old >> 32) == tag) {
+          e = (uint32_t)pos;
+          atomicOr(&a.ctl->shared_groups, 1u);
+          break;
+        }
+        pos = (pos + 1) & a.claim_mask;
+      }
+      a.ch.ent[g] = e;
+      a.ch.res[g] = kResUnresolved;
+    }
+  }
+}
+
 // The chunks of block-sized range vb (blockDim.x / 4 consecutive chunks); the
 // shared memory holds one region of group_bytes(kVerify) per group.  kAhead:
 // with the write-through of likely misses (written ahead of the pack step).
@@ -475,147 +647,11 @@ __device__ __forceinline__ void staged_range(const HashArgs& a, unsigned long lo
   if (ahead && lane == 0)  // the bytes past the last whole stripe
     for (uint32_t k = full; k < len; ++k) ahead_pk[k] = ahead_ar[k] = p[k];
 
-  unsigned long long h;
-  if (ns) {
-    const unsigned long long a0 = group_shfl(acc, gmask, gbase + 0);
-    const unsigned long long a1 = group_shfl(acc, gmask, gbase + 1);
-    const unsigned long long a2 = group_shfl(acc, gmask, gbase + 2);
-    const unsigned long long a3 = group_shfl(acc, gmask, gbase + 3);
-    h = xconverge(a0, a1, a2, a3);
-  } else {
-    h = kXP5;
-  }
-  h += len;
-  h = xfinish(h, p + full, len & 31);
-
-  if (a.fp_out != nullptr && lane == 0) a.fp_out[g] = h;
-  if (!kProbe) return;
-  // with a late wait, the cache's previous calls are complete from here on:
-  // the probe sees their inserts (candidates at or above slots_used are
-  // compared like any other), and every write of this kernel follows
-  unsigned long long slots_now = slots_used;
-  if (a.wait_late) {
-    pdl_wait();
-    slots_now = *reinterpret_cast<const volatile unsigned long long*>(&a.dstats[ST_SLOTS_USED]);
-  }
-
-  bool spec_equal = false;
-  if (speculate && hint_slot != kEmptySlot) {
-    unsigned long long dd = diff;
-    if (cmp && lane == 0)
-      for (uint32_t k = full; k < len; ++k) dd |= (unsigned long long)(p[k] ^ q[k]);
-    dd |= __shfl_xor_sync(gmask, dd, 1);
-    dd |= __shfl_xor_sync(gmask, dd, 2);
-    spec_equal = dd == 0;
-  }
-
-  const unsigned long long key = a.key16 ? (h & 0xFFFFULL) : h;
-  bool hit = false, cand = false;
-  uint32_t hit_slot = kEmptySlot;
-  if (slots_now) {
-    // The linear probe, in order.  A key+length candidate other than the
-    // verified hint is compared by the whole warp: each group walks its probe
-    // up to its next such candidate, then the warp compares the pending ones,
-    // one group's at a time, and the groups whose candidate differs walk on.
-    const unsigned wmask = present_lanes(vb, a.Ntot);
-    const uint32_t wl = threadIdx.x & 31, nl = __popc(wmask);
-    unsigned long long pos = mix64(key) & a.index_mask, probe = 0;
-    // the hinted slot holds these very bytes and this fingerprint: the index
-    // lists it under this key and length (both are written for every stored
-    // chunk), so it is the hit and the probe can be skipped
-    bool done = false;
-    if (spec_equal && hint_key == h) {
-      hit = true;
-      hit_slot = hint_slot;
-      done = true;
-    }
-    for (;;) {
-      uint32_t want = kEmptySlot;  // a candidate for the warp to compare
-      while (!done) {
-        if (probe > a.index_mask) {
-          done = true;
-          break;
-        }
-        const IndexEntry e = a.index[pos];
-        if (e.slot == kEmptySlot) {
-          done = true;
-          break;
-        }
-        pos = (pos + 1) & a.index_mask;
-        ++probe;
-        if (e.key == key && e.len == len) {
-          cand = true;
-          if (e.slot >= slots_now) {
-            if (lane == 0) atomicCAS(&a.ctl->err, 0, (int)GLEAM_ERR_INTERNAL);
-          } else if (e.slot == hint_slot) {
-            if (spec_equal) {
-              hit = true;
-              hit_slot = e.slot;
-              done = true;
-            }
-          } else {
-            want = e.slot;
-            break;
-          }
-        }
-      }
-      const unsigned pend = __ballot_sync(wmask, want != kEmptySlot) & 0x11111111u;
-      if (!pend) break;
-      for (unsigned m = pend; m; m &= m - 1) {
-        const int src = __ffs(m) - 1;
-        const uint8_t* ps = reinterpret_cast<const uint8_t*>(
-            __shfl_sync(wmask, reinterpret_cast<unsigned long long>(p), src));
-        const uint32_t slot = __shfl_sync(wmask, want, src);
-        const uint32_t ls = __shfl_sync(wmask, len, src);
-        const bool eq = lanes_equal<kMis>(ps, a.arena + (uint64_t)slot * a.C, ls, wmask, wl, nl);
-        if (gbase == src && eq) {
-          hit = true;
-          hit_slot = slot;
-          done = true;
-        }
-      }
-    }
-  }
-  if (lane == 0) {
-    a.ch.status[g] = hit ? kHit0 : (cand ? kMissCand : kMissNoCand);
-    a.ch.key[g] = h;  // the group key: the whole fingerprint
-    a.ch.len[g] = len;
-    a.ch.src[g] = (unsigned long long)p;
-    a.ch.pidx[g] = pid;
-    a.ch.hint[g] = hint;
-    if (kAhead) a.ch.spec[g] = ahead ? 1 : 0;
-    if (hit) {
-      a.ch.ent[g] = hit_slot;
-    } else if (kProbe && a.claim_tbl != nullptr) {
-      // the miss's (group key, length) entry of the per-call table, claimed
-      // with one 64-bit CAS that also stores a 32-bit tag of the pair (where
-      // the resolve kernel keeps a minimum): an entry found holding the same
-      // tag may be the chunk's group, which sends the call down the general
-      // path (shared_groups), where the groups are claimed again by the whole
-      // key; a different tag is another group's entry
-      const unsigned long long mixed = mix64(h ^ ((unsigned long long)len << 40));
-      const unsigned long long tag = mixed >> 32;
-      unsigned long long pos = mixed & a.claim_mask;
-      uint32_t e = 0xFFFFFFFFu;
-      for (unsigned long long probe = 0; probe <= a.claim_mask; ++probe) {
-        const unsigned long long old =
-            atomicCAS(reinterpret_cast<unsigned long long*>(&a.claim_tbl[pos]), 0ull,
-                      (tag << 32) | ((unsigned long long)g + 1ull));
-        if (old == 0) {
-          e = (uint32_t)pos;
-          break;
-        }
-        if ((old >> 32) == tag) {
-          e = (uint32_t)pos;
-          atomicOr(&a.ctl->shared_groups, 1u);
-          break;
-        }
-        pos = (pos + 1) & a.claim_mask;
-      }
-      a.ch.ent[g] = e;
-      a.ch.res[g] = kResUnresolved;
-    }
-  }
+  ChunkEnd e;
+  e.g = g, e.p = p, e.len = len, e.lane = lane, e.gbase = gbase, e.pid = pid;
+  e.acc = acc, e.hint = hint, e.hint_slot = hint_slot, e.hint_key = hint_key;
+  e.diff = diff, e.cmp = cmp, e.ahead = ahead, e.slots_used = slots_used;
+  record_chunk<kProbe, kAhead, kMis>(a, e, present_lanes(vb, a.Ntot));
 }
 
 }  // namespace
