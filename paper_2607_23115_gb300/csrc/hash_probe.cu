@@ -432,7 +432,10 @@ bool lone_call(const HashArgs& a) {
 
 template <bool kProbe, uint32_t kD>
 cudaError_t launch_lone(const HashArgs& a, uint32_t per, cudaStream_t s, bool pdl) {
-  const uint32_t smem = per * lone_bytes(kD);
+  // a call on its own asks for a full block's shared memory whatever its
+  // chunks, so that the few blocks spread over the SMs, two at most to each
+  // (300 chunks of 64 KiB, one to a block: 93 us the call, so 53)
+  const uint32_t smem = (a.wait_late ? per * lone_bytes(kD) : kLoneChunks * lone_bytes(4));
   cudaFuncSetAttribute((const void*)k_hash_lone<kProbe, kD>,
                        cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   return launch_kernel(k_hash_lone<kProbe, kD>, dim3((unsigned)((a.Ntot + per - 1) / per)),
