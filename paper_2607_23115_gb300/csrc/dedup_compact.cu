@@ -1597,51 +1597,26 @@ __device__ __forceinline__ void pack_publish(const DedupArgs& a, uint32_t G, uin
 //
 // A call of one payload that is launched chained (few enough chunks to leave
 // most of the GPU idle) runs its resolution, ranks, packing and publishing in
-// one launch.  Block b owns the contiguous chunks [b * per, (b + 1) * per),
-// at most one per thread.  Phase 1 classifies them and claims their (key,
-// length) groups without posting minima.  If no chunk of the call found its
-// group claimed by another (no in-call duplicate and no key collision: the
-// common case), every chunk that is not a cache hit is a miss of round one
-// (its own group's first chunk), so after one grid barrier each block knows
-// its misses' ranks from the blocks' counts, writes the outputs and inserts
-// its misses; after a second barrier every warp of the grid copies its share
-// of all misses' bytes (a block's own misses would leave the blocks that hold
-// the most of them as the call's tail).  Otherwise the general algorithm
+// one launch: k_resolve_direct if the hash kernel claimed the misses' (key,
+// length) groups as it recorded them, else (paper identifiers, and the
+// single-block small call) the steps below.  Block b owns the contiguous chunks
+// [b * per, (b + 1) * per), at most one per thread.  Phase 1 classifies them
+// and claims their groups without posting minima.  If no chunk of the call
+// found its group claimed by another (no in-call duplicate and no key
+// collision: the common case), every chunk that is not a cache hit is a miss of
+// round one (its own group's first chunk), so after one grid barrier each block
+// knows its misses' ranks from the blocks' counts, writes the outputs and
+// inserts its misses; after a second barrier every warp of the grid copies its
+// share of all misses' bytes (a block's own misses would leave the blocks that
+// hold the most of them as the call's tail).  Otherwise the general algorithm
 // takes over: the minima are posted and resolve_rank and pack_publish run on
 // the same grid.
 
-
-// Bit k of the result: byte k of w (k < 4) is not kHit0.
-__device__ __forceinline__ uint32_t not_hit_bits(uint32_t w) {
-  const uint32_t x = w ^ (0x01010101u * kHit0);
+// Bit k of the result: byte k of w (k < 4) is not v.
+__device__ __forceinline__ uint32_t bytes_not(uint32_t w, uint32_t v) {
+  const uint32_t x = w ^ (0x01010101u * v);
   const uint32_t t = (((x & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | x) & 0x80808080u;  // bit 8k+7: byte k != 0
   return ((t >> 7) & 1u) | ((t >> 14) & 2u) | ((t >> 21) & 4u) | ((t >> 28) & 8u);
-}
-
-// This thread's share of the call's chunks that are not cache hits: among
-// chunks [0, lim) (*below) and among all N (*all); the block's threads
-// together cover every chunk once.
-__device__ __forceinline__ void count_not_hit(const uint8_t* status, uint32_t N, uint32_t lim,
-                                              uint32_t* below, uint32_t* all) {
-  uint32_t b = 0, t = 0;
-  const bool vec = ((uintptr_t)status & 15) == 0;
-  for (uint32_t v = threadIdx.x; v * 16 < N; v += blockDim.x) {
-    const uint32_t b0 = v * 16;
-    uint32_t m = 0;
-    if (vec && b0 + 16 <= N) {
-      const uint4 q = __ldcg(reinterpret_cast<const uint4*>(status) + v);
-      m = not_hit_bits(q.x) | not_hit_bits(q.y) << 4 | not_hit_bits(q.z) << 8 |
-          not_hit_bits(q.w) << 12;
-    } else {
-      for (uint32_t k = 0; k < 16 && b0 + k < N; ++k)
-        m |= (uint32_t)(__ldcg(status + b0 + k) != kHit0) << k;
-    }
-    t += __popc(m);
-    const uint32_t nb = lim <= b0 ? 0u : min(lim - b0, 16u);
-    b += __popc(m & ((1u << nb) - 1u));
-  }
-  *below = b;
-  *all = t;
 }
 
 // The general algorithm on the one-launch kernel's grid, for a call with a
@@ -1706,15 +1681,11 @@ __device__ __forceinline__ void resolve_pack_fast(const DedupArgs& a, uint32_t G
   uint32_t len = 0, e = 0xFFFFFFFFu;
   unsigned long long key = 0, hint = 0;
   bool lead = false, stored = false, shared = false;
-  // the hash kernel claimed the groups: every miss is stored (the staged
-  // kernel marks no chunk uncached) and was given its entry there
-  const bool pre = a.pre_claimed != 0;
   if (valid) {
     // the chunk's record at once (one round trip, whatever its status)
     st = ch.status[g];
     const unsigned long long key0 = ch.key[g];
     const uint32_t len0 = ch.len[g];
-    const uint32_t ent0 = pre ? ch.ent[g] : 0u;
     hint = a.paper ? 0ull : ch.hint[g];
     if ((g & 31) == 0) P.mask[g >> 5] = 0;
     if (st == kHit0) {
@@ -1728,14 +1699,14 @@ __device__ __forceinline__ void resolve_pack_fast(const DedupArgs& a, uint32_t G
       key = key0;
       len = len0;
       bool claimed = true;
-      e = pre ? ent0 : group_entry(a, g, key, len, &claimed, true);
+      e = group_entry(a, g, key, len, &claimed, true);
       if (e == 0xFFFFFFFFu) {
         atomicCAS(&a.ctl->err, 0, (int)GLEAM_ERR_INTERNAL);
         ch.res[g] = kResLeader | 1u;
-      } else if (!pre) {
+      } else {
         ch.res[g] = kResUnresolved;
       }
-      if (!pre) ch.ent[g] = e;
+      ch.ent[g] = e;
       shared = !claimed;
       lead = stored = true;
     }
@@ -1747,38 +1718,21 @@ __device__ __forceinline__ void resolve_pack_fast(const DedupArgs& a, uint32_t G
     if (G > 1) atomicOr(&a.ctl->shared_groups, 1u);
   }
   bool ok = true;
-  unsigned long long pre_before = 0, pre_total = 0;
-  if (pre) {
-    // no barrier: every block counts the misses before its chunks, and in
-    // all, from the statuses the hash kernel wrote (at most 16 KiB of them)
-    uint32_t mb = 0, mt = 0;
-    count_not_hit(ch.status, N, bid * per, &mb, &mt);
-    pre_before = block_sum<unsigned long long>(mb, red64);
-    pre_total = block_sum<unsigned long long>(mt, red64);
-    if (threadIdx.x == 0) {
-      s_shared = (int)ldcg_u32(&a.ctl->shared_groups);
-      s_slots0 = my_slots0;
-      s_err = ld_volatile_s32(&a.ctl->err);
-    }
-    __syncthreads();
-    ok = s_err == 0;
-  } else {
-    if (G > 1 && threadIdx.x == 0) {
-      a.bcount[bid] = c_b;
-      a.bcount[G + bid] = s_b;
-    }
-    ok = grid_barrier(a.ctl, G, a.wait_ns, false);
-    if (threadIdx.x == 0) {
-      if (G > 1) s_shared = (int)ldcg_u32(&a.ctl->shared_groups);
-      s_slots0 = my_slots0;
-      s_err = G == 1 ? ld_volatile_s32(&a.ctl->err) : 0;
-    }
-    __syncthreads();
-    if (G == 1) ok = s_err == 0;  // a grid of one did not read the error word
+  if (G > 1 && threadIdx.x == 0) {
+    a.bcount[bid] = c_b;
+    a.bcount[G + bid] = s_b;
   }
+  ok = grid_barrier(a.ctl, G, a.wait_ns, false);
+  if (threadIdx.x == 0) {
+    if (G > 1) s_shared = (int)ldcg_u32(&a.ctl->shared_groups);
+    s_slots0 = my_slots0;
+    s_err = G == 1 ? ld_volatile_s32(&a.ctl->err) : 0;
+  }
+  __syncthreads();
+  if (G == 1) ok = s_err == 0;  // a grid of one did not read the error word
 
   if (s_shared) {
-    resolve_pack_general<kPlain>(a, G, bid, smem, ok, pre, valid && st != kHit0 && st != kUncached, e,
+    resolve_pack_general<kPlain>(a, G, bid, smem, ok, false, valid && st != kHit0 && st != kUncached, e,
                          key, len, g);
     return;
   }
@@ -1786,10 +1740,7 @@ __device__ __forceinline__ void resolve_pack_fast(const DedupArgs& a, uint32_t G
   // ---- 2: the fast path: ranks, outputs, inserts; then copies ----------------
   const unsigned long long slots0 = s_slots0;
   unsigned long long before = 0, total = c_b, sbefore = 0, stotal = s_b;
-  if (pre) {
-    before = sbefore = pre_before;
-    total = stotal = pre_total;
-  } else if (G > 1) {
+  if (G > 1) {
     unsigned long long b0 = 0, t0 = 0, sb0 = 0, st0 = 0;
     for (uint32_t j = threadIdx.x; j < G; j += kThreads) {
       const uint32_t v = ldcg_u32(&a.bcount[j]), sv = ldcg_u32(&a.bcount[G + j]);
@@ -2023,6 +1974,359 @@ __device__ __forceinline__ void resolve_pack_fast(const DedupArgs& a, uint32_t G
   finish_call(a, G, slots0, total, stotal, 0ull, 0ull, s_sum);
 }
 
+// The one-launch path where the hash kernel has claimed the misses' groups
+// (DedupArgs::pre_claimed; every miss is then stored).  If no group is shared,
+// every chunk that is not a cache hit is a miss, so every block reads the
+// statuses of the whole call (at most 16 KiB), turns them into a bit per chunk
+// with the misses counted before each word, and knows the rank of every miss,
+// the chunk of every rank, the hit mask and all of the call's counts: the
+// blocks write, copy and insert their shares and meet only at the end, to
+// publish.  What bounds it is the chain of round trips (statuses, claims or
+// copies, the arrival count, the publishing).
+constexpr uint32_t kDirectWords = 2 * kThreads;  // 32 chunks each
+
+struct DirectShared {
+  uint32_t bits[kDirectWords];  // chunk 32 w + k is not a cache hit: bit k of word w
+  uint16_t before[kDirectWords];  // such chunks before word w
+  unsigned long long scan[kWarps];
+  unsigned long long slots0;
+  int shared, err, last;
+};
+
+// Chunk of the r-th miss: the last of nw words with at most r misses before it,
+// then its bit.
+__device__ __forceinline__ uint32_t direct_miss(const DirectShared& sh, uint32_t nw, uint32_t r) {
+  uint32_t lo = 0, hi = nw;
+  while (hi - lo > 1) {
+    const uint32_t mid = (lo + hi) >> 1;
+    if (sh.before[mid] <= r) lo = mid;
+    else hi = mid;
+  }
+  uint32_t b = sh.bits[lo], k = r - sh.before[lo], pos = 0;
+#pragma unroll
+  for (uint32_t step = 16; step; step >>= 1) {
+    const uint32_t c = __popc(b & ((1u << step) - 1u));
+    if (k >= c) {
+      k -= c;
+      pos += step;
+      b >>= step;
+    }
+  }
+  return lo * 32 + pos;
+}
+
+template <bool kPlain>
+__device__ __forceinline__ void resolve_direct(const DedupArgs& a, uint32_t G, uint32_t bid,
+                                               uint8_t* smem) {
+  __shared__ DirectShared sh;
+  const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const ChunkArrays& ch = a.ch;
+  const PayloadDesc& P = a.one;
+  const uint32_t N = (uint32_t)a.Ntot, nw = (N + 31) / 32;
+  const uint32_t per = (N + G - 1) / G;  // <= kThreads (the host sizes the grid)
+  const uint32_t g = bid * per + threadIdx.x;
+  const bool valid = threadIdx.x < per && g < N;
+  if (threadIdx.x == 0) {
+    sh.slots0 = *(volatile const unsigned long long*)&a.dstats[ST_SLOTS_USED];
+    sh.shared = (int)ldcg_u32(&a.ctl->shared_groups);
+    sh.err = ld_volatile_s32(&a.ctl->err);
+    if (per > kThreads || nw > kDirectWords) atomicCAS(&a.ctl->err, 0, (int)GLEAM_ERR_INTERNAL);
+  }
+  // the thread's own chunk and its share of the statuses, in one round trip
+  unsigned long long key = 0, hint = 0;
+  uint32_t e = 0xFFFFFFFFu;
+  if (valid) {
+    key = ch.key[g];
+    hint = ch.hint[g];
+    e = ch.ent[g];
+  }
+  unsigned long long cnt = 0;  // misses of words < kThreads, of the others << 16, rejects << 32
+#pragma unroll
+  for (uint32_t k = 0; k < 2; ++k) {
+    const uint32_t word = k * kThreads + threadIdx.x, c0 = word * 32;
+    uint32_t m = 0, rej = 0;
+    if (c0 + 32 <= N) {
+      const uint4* q = reinterpret_cast<const uint4*>(ch.status + c0);
+      const uint4 v[2] = {__ldcg(q), __ldcg(q + 1)};
+#pragma unroll
+      for (uint32_t h = 0; h < 2; ++h) {
+        const uint32_t x[4] = {v[h].x, v[h].y, v[h].z, v[h].w};
+#pragma unroll
+        for (uint32_t u = 0; u < 4; ++u) {
+          m |= bytes_not(x[u], kHit0) << (16 * h + 4 * u);
+          rej += 4 - __popc(bytes_not(x[u], kMissCand));
+        }
+      }
+    } else {
+      for (uint32_t c = c0; c < N; ++c) {
+        const uint8_t st = __ldcg(ch.status + c);
+        m |= (uint32_t)(st != kHit0) << (c - c0);
+        rej += st == kMissCand;
+      }
+    }
+    sh.bits[word] = m;
+    cnt += (unsigned long long)__popc(m) << (16 * k) | (unsigned long long)rej << 32;
+  }
+  unsigned long long incl = cnt;
+#pragma unroll
+  for (uint32_t o = 1; o < 32; o <<= 1) {
+    const unsigned long long v = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += v;
+  }
+  if (lane == 31) sh.scan[w] = incl;
+  __syncthreads();
+  unsigned long long excl = incl - cnt, all = 0;
+#pragma unroll
+  for (uint32_t k = 0; k < kWarps; ++k) {
+    const unsigned long long v = sh.scan[k];
+    if (k < w) excl += v;
+    all += v;
+  }
+  const uint32_t total0 = (uint32_t)all & 0xFFFFu;
+  const uint32_t total = total0 + ((uint32_t)all >> 16);
+  sh.before[threadIdx.x] = (uint16_t)excl;
+  sh.before[kThreads + threadIdx.x] = (uint16_t)(total0 + (uint32_t)(excl >> 16 & 0xFFFFu));
+  __syncthreads();
+  const unsigned long long slots0 = sh.slots0;
+  bool ok = sh.err == 0;
+  const bool miss = valid && (sh.bits[g >> 5] >> (g & 31) & 1u);
+
+  if (sh.shared) {
+    // a group may be shared: the general algorithm, from cleared outputs
+    for (uint32_t k = bid * kThreads + threadIdx.x; k < nw; k += G * kThreads) P.mask[k] = 0;
+    if (bid == 0 && threadIdx.x == 0 && P.result) {
+      gleam_result_t* r = P.result;
+      r->n_miss = r->n_hit_cache = r->n_hit_intra = r->verify_rejects = r->miss_bytes = 0;
+    }
+    if (valid && !miss) ch.res[g] = kResHit0;
+    const uint32_t len = valid ? ch.len[g] : 0u;
+    resolve_pack_general<kPlain>(a, G, bid, smem, ok, true, miss, e, key, len, g);
+    return;
+  }
+
+  if (ok && total > a.nslots - slots0) {  // every block decides the same
+    if (threadIdx.x == 0) atomicCAS(&a.ctl->err, 0, (int)GLEAM_ERR_CAPACITY);
+    ok = false;
+  }
+  const unsigned long long last = (unsigned long long)(N - 1) * a.C;  // the last chunk's place
+  uint32_t n_spec = 0, n_spec_used = 0;
+  if (ok) {
+    // each miss records its slot and starts its index inserts (the first claim
+    // attempts), which complete after the copies below
+    const uint32_t r = miss ? sh.before[g >> 5] + __popc(sh.bits[g >> 5] & ((1u << (g & 31)) - 1u)) : 0u;
+    const unsigned long long slot = slots0 + r;
+    const uint32_t len = (uint32_t)min(a.C, P.n - (unsigned long long)min(g, N - 1) * a.C);
+    const bool ins_hint = miss && !a.paper && len >= kPrefixBytes;
+    PendingInsert pi{0ull, 0u}, ph{0ull, 0u};
+    if (miss) {
+      pi = index_insert_begin(a.index, a.index_mask, index_key(a, key), (uint32_t)slot);
+      if (ins_hint) ph = index_insert_begin(a.hints, a.index_mask, hint, (uint32_t)slot);
+      P.miss_idx[r] = g;
+      a.slot_len[slot] = len;
+      a.slot_key[slot] = key;
+    }
+    if (P.chunk_slot && valid) P.chunk_slot[g] = miss ? (uint32_t)slot : e;
+    for (uint32_t k = bid * kThreads + threadIdx.x; k < nw; k += G * kThreads)
+      P.mask[k] = ~sh.bits[k] & (k * 32 + 32 <= N ? 0xffffffffu : (1u << (N & 31)) - 1u);
+    if (a.spec_active && valid && ch.spec[g]) {
+      n_spec = 1;
+      n_spec_used = miss && r == g;
+    }
+    // every miss's bytes, in pieces of kPackPiece bytes spread over all the
+    // grid's warps (piece k of the miss of rank r is number r * ppc + k), all
+    // but those of misses the hash kernel already wrote where they belong
+    // (rank g means every earlier chunk is a miss)
+    const unsigned long long warps = (unsigned long long)G * kWarps;
+    const unsigned long long gw = (unsigned long long)bid * kWarps + w;
+    const unsigned long long ppc = (a.C + kPackPiece - 1) / kPackPiece;
+    const unsigned long long npieces = total * ppc;
+    const uint32_t wbase =
+        kPlain ? 0u : (uint32_t)__cvta_generic_to_shared(smem) + w * kPackWarpBytes;
+    const uint32_t bufs = wbase, bars = wbase + kPackBufs * kPackPiece;
+    PackMeta* meta =
+        reinterpret_cast<PackMeta*>(smem + w * kPackWarpBytes + kPackBufs * kPackPiece + 64);
+    PackRing ring{0u, 0u, 0u};
+    bool bulk_failed = false;
+    if constexpr (!kPlain) {
+      if (lane == 0) {
+        for (uint32_t b = 0; b < kPackBufs; ++b) mbar_init(bars + 8 * b);
+        mbar_fence_init();
+      }
+      __syncwarp();
+    }
+    auto copy_range = [&](unsigned long long lo, unsigned long long hi) {  // 32 pieces at a time
+      for (unsigned long long base = lo; base < hi; base += 32) {
+        const unsigned long long pc = base + lane;
+        uint32_t bytes = 0;
+        bool copy = false;
+        unsigned long long src = 0, d1 = 0, d2 = 0;
+        if (pc < hi) {
+          const uint32_t rr = (uint32_t)(pc / ppc);
+          const uint32_t off = (uint32_t)(pc - rr * ppc) * kPackPiece;
+          const uint32_t gg = direct_miss(sh, nw, rr);
+          const unsigned long long at = (unsigned long long)gg * a.C;
+          const uint32_t ln = (uint32_t)min(a.C, P.n - at);
+          if (off < ln && !(a.spec_active && rr == gg && ch.spec[gg])) {
+            bytes = min(kPackPiece, ln - off);
+            src = (unsigned long long)(P.buf + at + off);
+            d1 = (unsigned long long)(P.packed + rr * a.C + off);
+            d2 = (unsigned long long)(a.arena + (slots0 + rr) * a.C + off);
+            copy = true;
+          }
+        }
+        const unsigned cmask = __ballot_sync(0xffffffffu, copy);
+        if constexpr (!kPlain) {
+          const uint32_t at = __popc(cmask & ((1u << lane) - 1u));
+          if (copy) {
+            meta[at] = PackMeta{src, d1, d2, bytes, 0u};
+            // the pieces that wait for a buffer are on their way into L2
+            if (at >= kPackBufs && bytes >= 16) prefetch_l2(reinterpret_cast<const void*>(src), bytes & ~15u);
+          }
+          __syncwarp();
+          if (lane == 0 && cmask && !bulk_failed &&
+              !bulk_copy_batch(meta, __popc(cmask), bufs, bars, ring, a.wait_ns)) {
+            bulk_failed = true;
+            atomicCAS(&a.ctl->err, 0, (int)GLEAM_ERR_TIMEOUT);
+          }
+          if (copy) {  // the piece's last bytes % 16
+            const uint8_t* sp = reinterpret_cast<const uint8_t*>(src);
+            for (uint32_t k = bytes & ~15u; k < bytes; ++k)
+              reinterpret_cast<uint8_t*>(d1)[k] = reinterpret_cast<uint8_t*>(d2)[k] = sp[k];
+          }
+          __syncwarp();
+        } else {
+          for (unsigned todo = cmask; todo; todo &= todo - 1) {
+            const int j = __ffs(todo) - 1;
+            const unsigned long long sj = __shfl_sync(0xffffffffu, src, j);
+            const unsigned long long xj = __shfl_sync(0xffffffffu, d1, j);
+            const unsigned long long yj = __shfl_sync(0xffffffffu, d2, j);
+            const uint32_t lj = __shfl_sync(0xffffffffu, bytes, j);
+            warp_copy2(reinterpret_cast<uint8_t*>(xj), reinterpret_cast<uint8_t*>(yj),
+                       reinterpret_cast<const uint8_t*>(sj), lj, P);
+          }
+        }
+      }
+    };
+    if (a.copy_grab) {
+      // the pieces taken copy_grab at a time from a counter of the call, the
+      // warp's next grab requested before its current one is copied: warps
+      // on SMs that copy faster take more
+      const uint32_t grab = a.copy_grab;
+      uint32_t nxt = 0;
+      if (lane == 0) nxt = atomicAdd(&a.ctl->copy_next, grab);
+      nxt = __shfl_sync(0xffffffffu, nxt, 0);
+      while (nxt < npieces) {
+        uint32_t nn = 0;
+        if (lane == 0) nn = atomicAdd(&a.ctl->copy_next, grab);
+        copy_range(nxt, min(npieces, (unsigned long long)nxt + grab));
+        nxt = __shfl_sync(0xffffffffu, nn, 0);
+      }
+    } else {
+      copy_range(npieces * gw / warps, npieces * (gw + 1) / warps);
+    }
+    // each miss completes its inserts and frees the group entry it claimed,
+    // while the last pieces' stores are still in flight
+    if (miss) {
+      if (!index_insert_end(a.index, a.index_mask, index_key(a, key), (uint32_t)slot, len, pi,
+                            a.key16) ||
+          (ins_hint && !index_insert_end(a.hints, a.index_mask, hint, (uint32_t)slot, len, ph)))
+        atomicCAS(&a.ctl->err, 0, (int)GLEAM_ERR_INTERNAL);
+      if (e != 0xFFFFFFFFu) a.tbl[e] = CallEntry{0u, 0u};  // owner and the claim's tag
+      else atomicCAS(&a.ctl->err, 0, (int)GLEAM_ERR_INTERNAL);
+    }
+    if (!kPlain && lane == 0) bulk_wait_all<0>();  // every piece written before the block ends
+  }
+  if (a.spec_active) {
+    __shared__ unsigned long long red64[kWarps];
+    const unsigned long long b_spec = block_sum<unsigned long long>(n_spec, red64);
+    const unsigned long long b_used = block_sum<unsigned long long>(n_spec_used, red64);
+    if (threadIdx.x == 0) {
+      if (b_spec) atomicAdd(&a.ctl->spec_tried, b_spec);
+      if (b_used) atomicAdd(&a.ctl->spec_used, b_used);
+    }
+  }
+
+  // ---- the last block publishes -------------------------------------------------
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    sh.last = G == 1 || atomicAdd(&a.ctl->done, 1u) == G - 1;
+  }
+  __syncthreads();
+  if (!sh.last) return;
+  __threadfence();
+  const int err = ld_volatile_s32(&a.ctl->err);
+  if (err) {
+    clear_after_error(a);
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    const bool tail = sh.bits[nw - 1] >> ((N - 1) & 31) & 1u;  // the last chunk is a miss
+    const unsigned long long bytes =
+        (unsigned long long)total * a.C - (tail ? last + a.C - P.n : 0ull);
+    const unsigned long long rejects = all >> 32, hits = N - total;
+    if (a.spec_active || a.spec_state) {
+      const unsigned long long spec = __ldcg(&a.ctl->spec_tried);
+      if (err == 0 && a.spec_state) {
+        // automatic write-through: as in finish_call
+        uint32_t* st = a.spec_state;
+        if (spec) {
+          st[0] = 2 * __ldcg(&a.ctl->spec_used) >= spec ? 1u : 0u;
+          st[1] = 0;
+        } else if (st[0] == 0 && ++st[1] >= 256) {
+          st[0] = 1;
+          st[1] = 0;
+        }
+        *a.spec_mirror = st[0];
+      }
+      if (err == 0 && spec) atomicAdd(&a.dstats[ST_SPEC_CHUNKS], spec);
+      a.ctl->spec_tried = a.ctl->spec_used = 0;
+    }
+    if (err == 0) {
+      atomicAdd(&a.dstats[ST_CALLS], a.ncalls);
+      atomicAdd(&a.dstats[ST_CHUNKS], (unsigned long long)N);
+      if (hits) atomicAdd(&a.dstats[ST_HITS_CACHE], hits);
+      if (rejects) atomicAdd(&a.dstats[ST_REJECTS], rejects);
+      if (total) {
+        atomicAdd(&a.dstats[ST_MISSES], (unsigned long long)total);
+        atomicAdd(&a.dstats[ST_INSERTS], (unsigned long long)total);
+        a.dstats[ST_SLOTS_USED] = slots0 + total;
+        atomicAdd(&a.dstats[ST_BYTES_USED], bytes);
+      }
+    }
+    for (uint32_t k = 0; k < 2; ++k) {
+      gleam_result_t* t = k == 0 ? a.total : P.result;
+      if (!t) continue;
+      t->status = err;
+      t->n_miss = err ? 0 : total;
+      t->n_hit_cache = err ? 0 : hits;
+      t->n_hit_intra = 0;
+      t->verify_rejects = err ? 0 : rejects;
+      t->miss_bytes = err ? 0 : bytes;
+    }
+    // the control block as the next call expects it (no barrier was used)
+    DevCtl* c = a.ctl;
+    c->copy_next = 0;
+    c->err = 0;
+    c->shared_groups = 0;
+    c->done = 0;
+  }
+  __threadfence();
+}
+
+// Passes with this kernel against one in which the blocks exchanged the misses'
+// places through memory and a grid barrier: a Llama-3-8B layer, one call per
+// tensor, a tenth of its 64 KiB chunks changed, 575 -> 535 us (overlapping
+// calls 346 -> 314); 48 calls of 4 KiB-1 MiB 1,104 -> 1,067; one 64 MiB payload,
+// half of its 4 KiB chunks cached, 86.6 -> 81.4.
+template <bool kPlain>
+__global__ void __launch_bounds__(kThreads) k_resolve_direct(DedupArgs a) {
+  extern __shared__ __align__(128) uint8_t rd_smem[];
+  pdl_trigger();
+  pdl_wait();
+  resolve_direct<kPlain>(a, gridDim.x, blockIdx.x, rd_smem);
+}
+
 template <bool kPlain>
 __global__ void __launch_bounds__(kThreads) k_resolve_pack(DedupArgs a) {
   extern __shared__ __align__(128) uint8_t rp_smem[];
@@ -2226,8 +2530,10 @@ int pack_blocks_per_sm() { return blocks_per_sm(k_pack<false>, pack_smem_bytes(f
 // Co-resident blocks per SM of the one-launch resolve + pack kernel (its grid
 // barriers need every block of the grid resident at once).
 int resolve_pack_blocks_per_sm() {
-  return std::min(blocks_per_sm(k_resolve_pack<false>, pack_smem_bytes(false)),
-                  blocks_per_sm(k_resolve_pack<true>, pack_smem_bytes(true)));
+  return std::min({blocks_per_sm(k_resolve_pack<false>, pack_smem_bytes(false)),
+                   blocks_per_sm(k_resolve_pack<true>, pack_smem_bytes(true)),
+                   blocks_per_sm(k_resolve_direct<false>, pack_smem_bytes(false)),
+                   blocks_per_sm(k_resolve_direct<true>, pack_smem_bytes(true))});
 }
 
 // Co-resident blocks per SM for the cooperative launch (capped).
@@ -2255,7 +2561,9 @@ cudaError_t launch_dedup(const DedupArgs& a, int grid, int pack_grid, cudaStream
 }
 
 cudaError_t launch_resolve_pack(const DedupArgs& a, int grid, cudaStream_t s) {
-  auto kern = a.plain_copy ? k_resolve_pack<true> : k_resolve_pack<false>;
+  auto kern = a.pre_claimed
+                  ? (a.plain_copy ? k_resolve_direct<true> : k_resolve_direct<false>)
+                  : (a.plain_copy ? k_resolve_pack<true> : k_resolve_pack<false>);
   const uint32_t smem = pack_smem_bytes(a.plain_copy);
   cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   return launch_kernel(kern, dim3(grid), dim3(kThreads), smem, s, true, a);

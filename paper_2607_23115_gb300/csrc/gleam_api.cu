@@ -486,7 +486,7 @@ void note_call(gleam_cache* c, uint64_t Ntot) {
 // stream be launched as soon as all of its blocks have started, so that a
 // kernel's blocks are waiting on the GPU when the one before finishes instead
 // of being launched then.  After the hash kernel, a call of one payload runs
-// resolve, ranks, pack and publish as one launch (k_resolve_pack, one block
+// resolve, ranks, pack and publish as one launch (k_resolve_direct, one block
 // per 256 chunks or kChainBytesPerBlock of payload, at most kChainPackBlocks);
 // a batch runs the resolve kernel as a regular launch (a cooperative one is
 // never launched early) on at most kChainDedupBlocks blocks and the pack
@@ -751,13 +751,12 @@ int enqueue(gleam_cache* c, const gleam_payload_t* payloads, uint64_t count,
                                              (nbytes + per_block - 1) / per_block);
     rp_grid = (int)std::min<uint64_t>(std::max<uint64_t>(1, want), cap);
   }
-  // (a grid of one block needs no barrier before its ranks anyway)
   // overlapping calls give the one-launch kernel few blocks (a block per
   // kChainBytesPerBlock): its warps then share the copies out as they go
   // (Llama-3-8B, one call per tensor: +1%, four layers of it: +3%), where an
   // equal share per warp suits the one-block-per-SM grid of a call on its own
   if (one_launch && rp_grid > 1 && (c->flags & GLEAM_OVERLAP_CALLS)) d.copy_grab = kOverlapCopyGrab;
-  if (one_launch && rp_grid > 1 && hash_is_staged(h)) {
+  if (one_launch && hash_is_staged(h)) {
     h.claim_tbl = d.tbl;
     h.claim_mask = d.tbl_mask;
     d.pre_claimed = 1u;

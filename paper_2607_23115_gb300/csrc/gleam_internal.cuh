@@ -196,13 +196,13 @@ struct HashArgs {
   // speculative verify, the hint table and arena bytes of the slots counted as
   // used when it started, which no later call changes (no eviction).
   uint32_t wait_late;
-  // Calls resolved by the one-launch kernel on more than one block (one
-  // payload): the staged hash kernel claims each miss's entry in the per-call
-  // group table as it records the chunk (ent and res as the resolve kernel
-  // would set them; the entry's minv holds a tag of the chunk's (group key,
-  // length) until the resolve kernel frees it; shared_groups if an entry with
-  // the same tag was found), so that the resolve kernel needs no claims and
-  // no barrier before its ranks.  Null: no claims here.
+  // Calls resolved by the one-launch kernel (one payload): the hash kernel
+  // claims each miss's entry in the per-call group table as it records the
+  // chunk (ent and res as the resolve kernel would set them; the entry's minv
+  // holds a tag of the chunk's (group key, length) until the resolve kernel
+  // frees it; shared_groups if an entry with the same tag was found), so that
+  // the resolve kernel needs no claims and no barrier before its ranks.  Null:
+  // no claims here.
   CallEntry* claim_tbl;
   unsigned long long claim_mask;
   unsigned long long wait_ns;  // limit of every wait between the warps of a block
@@ -291,7 +291,7 @@ cudaError_t load_hash_kernels();
 cudaError_t launch_dedup(const DedupArgs& a, int grid, int pack_grid, cudaStream_t s,
                          bool pdl = false);
 // Resolve, rank, pack and publish of a one-payload call in one launch on
-// `grid` blocks (see k_resolve_pack), with programmatic stream serialization.
+// `grid` blocks (k_resolve_direct, or k_resolve_pack without claims), with programmatic stream serialization.
 cudaError_t launch_resolve_pack(const DedupArgs& a, int grid, cudaStream_t s);
 // A whole call (hash, resolve and rank, pack) as one single-block kernel, for
 // calls with few chunks outside GLEAM_PAPER_IDS mode; the block hashes
