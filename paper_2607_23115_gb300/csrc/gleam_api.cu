@@ -489,9 +489,9 @@ void note_call(gleam_cache* c, uint64_t Ntot) {
 // resolve, ranks, pack and publish as one launch (k_resolve_direct, one block
 // per 256 chunks or kChainBytesPerBlock of payload, at most kChainPackBlocks);
 // a batch runs the resolve kernel as a regular launch (a cooperative one is
-// never launched early) on at most kChainDedupBlocks blocks and the pack
-// kernel on at most kChainPackBlocks: every waiting block holds its SM
-// resources.  With GLEAM_OVERLAP_CALLS the hash kernel also fingerprints
+// never launched early) and the pack kernel; where calls overlap on at most
+// kChainDedupBlocks and kChainPackBlocks blocks: every waiting block holds its
+// SM resources.  With GLEAM_OVERLAP_CALLS the hash kernel also fingerprints
 // before it waits (HashArgs::wait_late).  Evicting caches and the test hook
 // that makes a block skip a barrier keep the plain launches.
 #ifndef GLEAM_CHAIN_MAX_CHUNKS
@@ -511,6 +511,7 @@ constexpr uint64_t kChainMaxChunks = GLEAM_CHAIN_MAX_CHUNKS;
 constexpr uint64_t kChainMaxBytes = 256ull << 20;
 constexpr int kChainDedupBlocks = GLEAM_CHAIN_DEDUP_BLOCKS;
 constexpr int kChainPackBlocks = GLEAM_CHAIN_PACK_BLOCKS;
+constexpr uint64_t kChainDedupBytes = 2ull << 20;
 // Overlapping calls: a block of the one-launch kernel per 2 MiB of payload
 // (Llama-3-8B, one call per tensor: 1,558-1,571 GB/s, against 1,480-1,495
 // with 1 MiB), or per 512 KiB for calls under 4 MiB, whose copies would
@@ -782,9 +783,20 @@ int enqueue(gleam_cache* c, const gleam_payload_t* payloads, uint64_t count,
     int pgrid = pack_grid(c, Ntot, nbytes);
     if (chain) {
       // one chunk per thread of the resolve kernel: a call of at most 256
-      // chunks resolves in one block, without any grid-wide barrier
-      grid = (int)std::min<uint64_t>(kChainDedupBlocks, (Ntot + 255) / 256);
-      pgrid = std::min(pgrid, kChainPackBlocks);
+      // chunks resolves in one block, without any grid-wide barrier.  Calls
+      // that overlap keep to few blocks, which wait for each other's calls; a
+      // batch on its own takes a block per kChainDedupBytes too, at most one
+      // per SM, and a full wave to copy (40 payloads, 260 MB, 15,870 chunks, a
+      // tenth of them changed: 244 -> 228 us; one block per 512 KiB up to
+      // three per SM, 229 us, and a 52 MB batch 76 -> 83)
+      if (c->flags & GLEAM_OVERLAP_CALLS) {
+        grid = (int)std::min<uint64_t>(kChainDedupBlocks, (Ntot + 255) / 256);
+        pgrid = std::min(pgrid, kChainPackBlocks);
+      } else {
+        grid = (int)std::min<uint64_t>(
+            c->coop_max_blocks / GLEAM_SOLO_CAP_DIV,
+            std::max<uint64_t>((Ntot + 255) / 256, nbytes / kChainDedupBytes));
+      }
     }
     if (one_launch) {
       rc = cuda_err(launch_resolve_pack(d, rp_grid, s));
