@@ -597,18 +597,22 @@ __device__ __forceinline__ uint32_t block_rank(bool f, uint32_t* cnt, uint32_t* 
   return r;
 }
 
-// Selects and removes the K victims; false if a grid barrier failed.
-__device__ bool lru_evict(const DedupArgs& a, uint32_t G, uint32_t bid,
-                          unsigned long long slots0, unsigned long long K,
-                          unsigned long long* sred, uint32_t* cnt, uint32_t* off,
-                          unsigned long long* red64) {
+// The cut-off stamp by a two-pass radix select on its high and low 16 bits, and
+// how many candidates at it are victims; false if a grid barrier failed.  Out
+// of line: for stamps that lru_evict's one pass by age does not tell apart.
+// The bins hold that pass's counts.
+__device__ __noinline__ bool lru_radix_cut(const DedupArgs& a, uint32_t G, uint32_t bid,
+                                           unsigned long long slots0, unsigned long long K,
+                                           unsigned long long* sred, uint32_t* off,
+                                           uint32_t* cut, unsigned long long* ties) {
   static_assert(kLruBins == kThreads * kThreads, "one part of kThreads bins per thread");
   const uint32_t lane = threadIdx.x & 31;
   const unsigned long long tid = (unsigned long long)bid * kThreads + threadIdx.x;
   const unsigned long long nth = (unsigned long long)G * kThreads;
   const uint32_t now = a.epoch;
-
-  // cut-off stamp: radix select on the high, then the low 16 bits
+  if (!grid_barrier(a.ctl, G, a.wait_ns, false)) return false;  // every block has read the bins
+  for (unsigned long long q = tid; q < kLruBins; q += nth) a.bins[q] = 0u;
+  if (!grid_barrier(a.ctl, G, a.wait_ns, false)) return false;
   uint32_t hi_bin = 0;
   unsigned long long below = 0;
   for (int pass = 0; pass < 2; ++pass) {
@@ -673,8 +677,104 @@ __device__ bool lru_evict(const DedupArgs& a, uint32_t G, uint32_t bid,
     hi_bin = __ldcg(&a.ctl->lru_hi);
     below = __ldcg(&a.ctl->lru_below);
   }
-  const uint32_t cut = __ldcg(&a.ctl->lru_cut);
-  const unsigned long long ties = __ldcg(&a.ctl->lru_ties);
+  *cut = __ldcg(&a.ctl->lru_cut);
+  *ties = __ldcg(&a.ctl->lru_ties);
+  return true;
+}
+
+// Ages (calls since the last use) that have a bin of their own; bin 0 holds
+// stamps later than this call's (the clock was set back), the last bin all
+// greater ages.  Bin b is word b + kAgeBase: the sixteen bins of a thread
+// (lru_evict) are then four 16-byte loads.
+constexpr uint32_t kAgeBins = 16 * kThreads;
+constexpr uint32_t kAgeBase = 3;
+static_assert(kAgeBins + kAgeBase < kLruBins, "the bins' array holds them");
+
+// Selects and removes the K victims; false if a grid barrier failed.
+__device__ bool lru_evict(const DedupArgs& a, uint32_t G, uint32_t bid,
+                          unsigned long long slots0, unsigned long long K,
+                          unsigned long long* sred, uint32_t* cnt, uint32_t* off,
+                          unsigned long long* red64) {
+  const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const unsigned long long tid = (unsigned long long)bid * kThreads + threadIdx.x;
+  const unsigned long long nth = (unsigned long long)G * kThreads;
+  const uint32_t now = a.epoch;
+
+  // The cut-off stamp: one histogram of the candidates' ages, from which every
+  // block finds the bin of the K-th oldest.  A warp adds up a run of slots of
+  // one age before it touches the bin.
+  {
+    uint32_t run = 0xFFFFFFFFu, run_cnt = 0;
+    for (unsigned long long base = tid - lane; base < slots0; base += nth) {
+      const unsigned long long sl = base + lane;
+      uint32_t bin = 0xFFFFFFFFu;
+      if (sl < slots0) {
+        const uint32_t u = __ldcg(&a.last_use[sl]);
+        if (u != now) bin = u > now ? 0u : min(now - u, kAgeBins);
+      }
+      const unsigned have = __ballot_sync(0xffffffffu, bin != 0xFFFFFFFFu);
+      if (!have) continue;
+      const uint32_t b0 = __shfl_sync(0xffffffffu, bin, __ffs(have) - 1);
+      if (__ballot_sync(0xffffffffu, bin == b0) == have) {
+        if (b0 != run) {
+          if (run_cnt && lane == 0) atomicAdd(&a.bins[kAgeBase + run], run_cnt);
+          run = b0;
+          run_cnt = 0;
+        }
+        run_cnt += __popc(have);
+      } else {
+        const unsigned peers = __match_any_sync(0xffffffffu, bin);
+        if (bin != 0xFFFFFFFFu && lane == (uint32_t)(__ffs(peers) - 1))
+          atomicAdd(&a.bins[kAgeBase + bin], (uint32_t)__popc(peers));
+      }
+    }
+    if (run_cnt && lane == 0) atomicAdd(&a.bins[kAgeBase + run], run_cnt);
+  }
+  if (!grid_barrier(a.ctl, G, a.wait_ns, false)) return false;
+  uint32_t cut = 0;
+  unsigned long long ties = 0;
+  {
+    // thread i: the bins of ages kAgeBins - 16 i down to kAgeBins - 16 i - 15
+    uint32_t v[16], sum = 0;
+    const uint4* b4 = reinterpret_cast<const uint4*>(a.bins + kAgeBase + kAgeBins -
+                                                     16 * threadIdx.x - 15);
+#pragma unroll
+    for (uint32_t k = 0; k < 4; ++k) {
+      const uint4 x = __ldcg(b4 + k);
+      v[4 * k] = x.x, v[4 * k + 1] = x.y, v[4 * k + 2] = x.z, v[4 * k + 3] = x.w;
+      sum += x.x + x.y + x.z + x.w;
+    }
+    uint32_t incl = sum;
+#pragma unroll
+    for (uint32_t o = 1; o < 32; o <<= 1) {
+      const uint32_t x = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += x;
+    }
+    if (lane == 31) cnt[w] = incl;
+    if (threadIdx.x == 0) off[0] = 0;  // the bin of the K-th oldest; 0: in no thread's
+    __syncthreads();
+    unsigned long long older = incl - sum;
+    for (uint32_t k = 0; k < w; ++k) older += cnt[k];
+    if (older < K && K <= older + sum) {
+#pragma unroll
+      for (uint32_t k = 0; k < 16; ++k) {
+        const uint32_t c = v[15 - k];
+        if (older < K && K <= older + c) {
+          off[0] = kAgeBins - 16 * threadIdx.x - k;
+          sred[0] = K - older;
+        }
+        older += c;
+      }
+    }
+    __syncthreads();
+    const uint32_t bin = off[0];
+    cut = now - bin;
+    ties = sred[0];
+    __syncthreads();
+    if (bin == 0 || bin == kAgeBins) {
+      if (!lru_radix_cut(a, G, bid, slots0, K, sred, off, &cut, &ties)) return false;
+    }
+  }
 
   // per contiguous slot range: candidates older than the cut-off, and at it
   const unsigned long long per = ((slots0 + G - 1) / G + 31) & ~31ull;
@@ -697,6 +797,8 @@ __device__ bool lru_evict(const DedupArgs& a, uint32_t G, uint32_t bid,
     }
   }
   if (!grid_barrier(a.ctl, G, a.wait_ns, false)) return false;
+  // every block has read the ages' bins
+  for (unsigned long long q = tid; q <= kAgeBase + kAgeBins; q += nth) a.bins[q] = 0u;
   {
     unsigned long long tie_before = 0, lt_before = 0;
     for (uint32_t j = threadIdx.x; j < bid; j += kThreads) {
@@ -727,23 +829,52 @@ __device__ bool lru_evict(const DedupArgs& a, uint32_t G, uint32_t bid,
   }
   if (!grid_barrier(a.ctl, G, a.wait_ns, false)) return false;
 
-  // the victims' entries leave the index and the hint table
+  // the victims' entries leave the index and the hint table; kTabWays entries
+  // of each per thread at a time, so that their loads wait together
+  constexpr uint32_t kTabWays = 4;
   const unsigned long long tsize = a.index_mask + 1;
-  for (unsigned long long q = tid; q < tsize; q += nth) {
-    const uint32_t s1 = a.index[q].slot;
-    if (s1 < slots0 && a.vflag[s1]) a.index[q].slot = kTombSlot;
-    const uint32_t s2 = a.hints[q].slot;
-    if (s2 < slots0 && a.vflag[s2]) a.hints[q].slot = kTombSlot;
+  for (unsigned long long q0 = tid; q0 < tsize; q0 += kTabWays * nth) {
+    uint32_t s1[kTabWays], s2[kTabWays];
+#pragma unroll
+    for (uint32_t k = 0; k < kTabWays; ++k) {
+      const unsigned long long q = q0 + k * nth;
+      s1[k] = q < tsize ? a.index[q].slot : kEmptySlot;
+      s2[k] = q < tsize ? a.hints[q].slot : kEmptySlot;
+    }
+    bool f1[kTabWays], f2[kTabWays];
+#pragma unroll
+    for (uint32_t k = 0; k < kTabWays; ++k) {
+      f1[k] = s1[k] < slots0 && a.vflag[s1[k]];
+      f2[k] = s2[k] < slots0 && a.vflag[s2[k]];
+    }
+#pragma unroll
+    for (uint32_t k = 0; k < kTabWays; ++k) {
+      const unsigned long long q = q0 + k * nth;
+      if (f1[k]) a.index[q].slot = kTombSlot;
+      if (f2[k]) a.hints[q].slot = kTombSlot;
+    }
   }
   if (!grid_barrier(a.ctl, G, a.wait_ns, false)) return false;
-  for (unsigned long long q = tid; q < tsize; q += nth) {
-    const unsigned long long prev = (q + tsize - 1) & a.index_mask;
-    if (a.index[q].slot != kEmptySlot && a.index[prev].slot == kEmptySlot)
-      compact_cluster(a.index, a.index_mask, q);
-    if (a.hints[q].slot != kEmptySlot && a.hints[prev].slot == kEmptySlot)
-      compact_cluster(a.hints, a.index_mask, q);
+  for (unsigned long long q0 = tid; q0 < tsize; q0 += kTabWays * nth) {
+    bool f1[kTabWays], f2[kTabWays];  // a cluster begins here
+#pragma unroll
+    for (uint32_t k = 0; k < kTabWays; ++k) {
+      const unsigned long long q = q0 + k * nth;
+      f1[k] = f2[k] = false;
+      if (q < tsize) {
+        const unsigned long long prev = (q + tsize - 1) & a.index_mask;
+        f1[k] = a.index[q].slot != kEmptySlot && a.index[prev].slot == kEmptySlot;
+        f2[k] = a.hints[q].slot != kEmptySlot && a.hints[prev].slot == kEmptySlot;
+      }
+    }
+#pragma unroll 1
+    for (uint32_t k = 0; k < kTabWays; ++k) {
+      if (f1[k]) compact_cluster(a.index, a.index_mask, q0 + k * nth);
+      if (f2[k]) compact_cluster(a.hints, a.index_mask, q0 + k * nth);
+    }
   }
   if (!grid_barrier(a.ctl, G, a.wait_ns, false)) return false;
+#pragma unroll 4
   for (unsigned long long q = tid; q < tsize; q += nth) {
     if (a.index[q].slot == kTombSlot) a.index[q].slot = kEmptySlot;
     if (a.hints[q].slot == kTombSlot) a.hints[q].slot = kEmptySlot;

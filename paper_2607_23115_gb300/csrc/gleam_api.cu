@@ -65,6 +65,7 @@ struct gleam_cache {
   gleam_result_t* h_result = nullptr;      // page-locked, mapped: gleam_dedup_copy's result
   gleam_result_t* h_result_dev = nullptr;  // its device address
   int coop_max_blocks = 0;
+  int coop_per_sm = 1;      // of those, to each SM
   int pack_max_blocks = 0;  // pack kernel: all co-resident blocks
   int rp_max_blocks = 0;    // one-launch resolve + pack: all co-resident blocks
   cudaEvent_t done = nullptr;
@@ -428,11 +429,38 @@ int describe(gleam_cache* c, PtrChecker& chk, const gleam_payload_t& p, PayloadD
 // kBytesPerDedupBlock of payload), at most the co-resident maximum.
 constexpr uint64_t kBytesPerDedupBlock = 256ull << 10;
 
+// At most a block per SM where calls share the GPU or barriers are most of the
+// kernel's time.
+int one_per_sm(const gleam_cache* c) { return c->coop_max_blocks / c->coop_per_sm; }
+
+// Blocks that an eviction wants, for a call that may evict (else 1): it passes
+// over the whole index three times, kEvictEntries entries of it to a block (54
+// calls of 1.6 MB in all, 30% of it evicted: 6.1 ms with one block each, 4.1
+// with 8,192 entries to a block, 3.1 with 512, 3.0 with 256), on at most a
+// block per SM.
+constexpr uint64_t kEvictEntries = 256;
+int evict_grid(const gleam_cache* c, uint64_t nchunks) {
+  if (!(c->flags & GLEAM_EVICT_LRU) || c->slots_bound + nchunks <= c->nslots) return 1;
+  return (int)std::max<uint64_t>(
+      1, std::min<uint64_t>(one_per_sm(c), c->index_cap / kEvictEntries));
+}
+
+// A call that evicts passes five more grid barriers: up to kEvictFewChunks
+// chunks and kEvictFewBytes, it takes at most a block per SM for all of them (a
+// batch of 6,658 chunks, 436 MB, a tenth of it evicted: 278 us with three per
+// SM, 274 with two, 257 with one); beyond, its in-call duplicates may be most
+// of the work (1 GiB of 64 KiB chunks, half of them copies: 735 us with three
+// per SM, 821 with one).
+constexpr uint64_t kEvictFewChunks = 8192, kEvictFewBytes = 512ull << 20;
+
 int dedup_grid(const gleam_cache* c, uint64_t nchunks, uint64_t nbytes) {
   const uint64_t per_block = dedup_chunks_per_block();
   const uint64_t want = std::max<uint64_t>((nchunks + per_block - 1) / per_block,
                                            (nbytes + kBytesPerDedupBlock - 1) / kBytesPerDedupBlock);
-  return (int)std::max<uint64_t>(1, std::min<uint64_t>(c->coop_max_blocks, want));
+  const int evict = evict_grid(c, nchunks);
+  const uint64_t most = evict > 1 && nchunks <= kEvictFewChunks && nbytes <= kEvictFewBytes
+                            ? one_per_sm(c) : c->coop_max_blocks;
+  return (int)std::max<uint64_t>(evict, std::min<uint64_t>(most, std::max<uint64_t>(1, want)));
 }
 
 // Blocks of the pack kernel: one per 256 chunks or per kBytesPerPackBlock of
@@ -492,8 +520,8 @@ void note_call(gleam_cache* c, uint64_t Ntot) {
 // never launched early) and the pack kernel; where calls overlap on at most
 // kChainDedupBlocks and kChainPackBlocks blocks: every waiting block holds its
 // SM resources.  With GLEAM_OVERLAP_CALLS the hash kernel also fingerprints
-// before it waits (HashArgs::wait_late).  Evicting caches and the test hook
-// that makes a block skip a barrier keep the plain launches.
+// before it waits (HashArgs::wait_late; not for evicting caches).  The test hook
+// that makes a block skip a barrier keeps the plain launches.
 #ifndef GLEAM_CHAIN_MAX_CHUNKS
 #define GLEAM_CHAIN_MAX_CHUNKS 16384
 #endif
@@ -529,9 +557,6 @@ constexpr uint64_t kChainBytesPerBlock = GLEAM_CHAIN_BYTES_PER_BLOCK;
 #ifndef GLEAM_SOLO_KIB_PER_BLOCK
 #define GLEAM_SOLO_KIB_PER_BLOCK 512
 #endif
-#ifndef GLEAM_SOLO_CAP_DIV
-#define GLEAM_SOLO_CAP_DIV 3
-#endif
 constexpr uint64_t kSoloBytesPerBlock = (uint64_t)GLEAM_SOLO_KIB_PER_BLOCK << 10;
 #ifndef GLEAM_OVERLAP_COPY_GRAB
 #define GLEAM_OVERLAP_COPY_GRAB 8
@@ -541,8 +566,7 @@ constexpr uint32_t kOverlapCopyGrab = GLEAM_OVERLAP_COPY_GRAB;
 static_assert(kChainMaxChunks <= (uint64_t)kChainPackBlocks * 256, "chain limit");
 
 bool chain_call(const gleam_cache* c, uint64_t Ntot, uint64_t nbytes, int skip_block) {
-  return Ntot <= kChainMaxChunks && nbytes <= kChainMaxBytes && skip_block < 0 &&
-         !(c->flags & GLEAM_EVICT_LRU);
+  return Ntot <= kChainMaxChunks && nbytes <= kChainMaxBytes && skip_block < 0;
 }
 
 // Orders a call on stream s after the cache's previous work: an event wait,
@@ -730,13 +754,15 @@ int enqueue(gleam_cache* c, const gleam_payload_t* payloads, uint64_t count,
   // overlapping calls: the staged hash kernels fingerprint before they wait
   // (others ignore the field and wait first); the write-through stays off, as
   // it writes arena slots counted from a slot count that may still change
-  h.wait_late = chain && (c->flags & GLEAM_OVERLAP_CALLS) && !(c->flags & GLEAM_PAPER_IDS) ? 1u : 0u;
+  h.wait_late = chain && (c->flags & GLEAM_OVERLAP_CALLS) &&
+                        !(c->flags & (GLEAM_PAPER_IDS | GLEAM_EVICT_LRU))
+                    ? 1u : 0u;
   // host payloads too: a chunk written ahead then spares the pack a second
   // read over the CPU-GPU link (managed memory stays out)
   set_spec(c, &h, &d, aligned && packed_aligned && !chk.saw_managed() && !h.wait_late);
   // a payload resolved by the one-launch kernel: its staged hash kernel
   // claims the misses' groups as it records them
-  const bool one_launch = !fused && chain && count == 1 && !d.classes;
+  const bool one_launch = !fused && chain && count == 1 && !d.classes && !d.lru;
   int rp_grid = 1;
   if (one_launch) {
     // at most one chunk per thread, and one block per kChainBytesPerBlock of
@@ -746,7 +772,7 @@ int enqueue(gleam_cache* c, const gleam_payload_t* payloads, uint64_t count,
         solo || nbytes < kChainSmallCall ? kSoloBytesPerBlock : kChainBytesPerBlock;
     const uint64_t cap =
         solo ? (uint64_t)std::min(c->rp_max_blocks,
-                                  std::max(kChainPackBlocks, c->coop_max_blocks / GLEAM_SOLO_CAP_DIV))
+                                  std::max(kChainPackBlocks, one_per_sm(c)))
              : (uint64_t)kChainPackBlocks;
     const uint64_t want = std::max<uint64_t>((Ntot + dedup_threads() - 1) / dedup_threads(),
                                              (nbytes + per_block - 1) / per_block);
@@ -794,9 +820,10 @@ int enqueue(gleam_cache* c, const gleam_payload_t* payloads, uint64_t count,
         pgrid = std::min(pgrid, kChainPackBlocks);
       } else {
         grid = (int)std::min<uint64_t>(
-            c->coop_max_blocks / GLEAM_SOLO_CAP_DIV,
+            one_per_sm(c),
             std::max<uint64_t>((Ntot + 255) / 256, nbytes / kChainDedupBytes));
       }
+      grid = std::max(grid, evict_grid(c, Ntot));
     }
     if (one_launch) {
       rc = cuda_err(launch_resolve_pack(d, rp_grid, s));
@@ -909,6 +936,7 @@ int gleam_cache_create_ex(size_t capacity_bytes, size_t chunk_bytes, uint32_t fl
     step(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device));
     const int per_sm = dedup_blocks_per_sm();
     c->coop_max_blocks = sms * per_sm;
+    c->coop_per_sm = std::max(1, per_sm);
     c->pack_max_blocks = sms * pack_blocks_per_sm();
     c->rp_max_blocks = sms * resolve_pack_blocks_per_sm();
     c->small_max_chunks = small_call_groups();
