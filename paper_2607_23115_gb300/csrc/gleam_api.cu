@@ -751,6 +751,8 @@ int enqueue(gleam_cache* c, const gleam_payload_t* payloads, uint64_t count,
   }
   const bool fused = small_call(c, Ntot, nbytes, d.skip_block);
   const bool chain = chain_call(c, Ntot, nbytes, d.skip_block);
+  // a larger call on its own chains its launches too, on its full grids
+  const bool pdl = chain || (d.skip_block < 0 && !(c->flags & GLEAM_OVERLAP_CALLS));
   // overlapping calls: the staged hash kernels fingerprint before they wait
   // (others ignore the field and wait first); the write-through stays off, as
   // it writes arena slots counted from a slot count that may still change
@@ -804,7 +806,7 @@ int enqueue(gleam_cache* c, const gleam_payload_t* payloads, uint64_t count,
     if ((rc = cuda_err(launch_small_call(h, d, aligned, s, chain))) != GLEAM_OK) return rc;
     if (ev[1]) cudaEventRecord(ev[1], s);
   } else {
-    if ((rc = cuda_err(launch_hash(h, aligned, s, chain))) != GLEAM_OK) return rc;
+    if ((rc = cuda_err(launch_hash(h, aligned, s, pdl))) != GLEAM_OK) return rc;
     if (ev[1]) cudaEventRecord(ev[1], s);
     int pgrid = pack_grid(c, Ntot, nbytes);
     if (chain) {
@@ -828,7 +830,7 @@ int enqueue(gleam_cache* c, const gleam_payload_t* payloads, uint64_t count,
     if (one_launch) {
       rc = cuda_err(launch_resolve_pack(d, rp_grid, s));
     } else {
-      rc = cuda_err(launch_dedup(d, grid, pgrid, s, chain));
+      rc = cuda_err(launch_dedup(d, grid, pgrid, s, pdl));
     }
     if (rc != GLEAM_OK) {
       cudaMemsetAsync(c->ctl, 0, sizeof(DevCtl), s);  // the hash kernel may have flagged it
