@@ -471,11 +471,15 @@ __device__ uint32_t group_entry(const DedupArgs& a, uint32_t g, unsigned long lo
   for (uint64_t probe = 0; probe <= a.tbl_mask; ++probe) {
     uint32_t o = cas_first && probe == 0 ? 0u : ldcg_u32(&a.tbl[pos].owner);
     if (o == 0) {
-      o = atomicCAS(&a.tbl[pos].owner, 0u, g + 1);
-      if (o == 0) {
+      // a free entry is all zeros: the claim posts the claimant's minimum too
+      const unsigned long long old =
+          atomicCAS(reinterpret_cast<unsigned long long*>(&a.tbl[pos]), 0ull,
+                    (unsigned long long)~g << 32 | (unsigned long long)(g + 1));
+      if (old == 0) {
         if (claimed) *claimed = true;
         return (uint32_t)pos;
       }
+      o = (uint32_t)old;
     }
     if (a.ch.key[o - 1] == k && a.ch.len[o - 1] == len) {
       if (claimed) *claimed = false;
@@ -943,8 +947,20 @@ __device__ __forceinline__ void resolve_rank(const DedupArgs& a, uint32_t G, uin
   const unsigned long long my_slots0 =
       threadIdx.x == 0 ? *(volatile const unsigned long long*)&a.dstats[ST_SLOTS_USED] : 0ull;
 
+  // contiguous chunk range of each block, for the ranks
+  const uint64_t per = (((uint64_t)N + G - 1) / G + 31) & ~31ull;
+  const uint32_t lo = (uint32_t)min((uint64_t)N, bid * per);
+  const uint32_t hi = (uint32_t)min((uint64_t)N, lo + per);
+  // the rounds count the misses of every range as they find them (a warp step's
+  // 32 chunks lie in one range), so that the ranks need no counting pass and no
+  // barrier after it; a grid of one, and KEY16 classes, whose rejects wait for
+  // every miss's class, count them afterwards
+  const bool counted = !claimed && !a.classes && G > 1;
+
   // ---- A: clear outputs, round-1 claims; LRU: stamp the slots hit ----------
   if (!claimed) {
+    if (counted)
+      for (uint32_t j = tid; j < 2 * G; j += nth) a.bcount[j] = 0;
     unsigned long long distinct = 0;
     for (uint32_t p = tid; p < a.count; p += nth) {
       gleam_result_t* r = desc(a, p).result;
@@ -980,7 +996,8 @@ __device__ __forceinline__ void resolve_rank(const DedupArgs& a, uint32_t G, uin
           ch.ent[g] = 0xFFFFFFFFu;
           ch.res[g] = kResLeader | kResNoSlot | 1u;
         } else {
-          const uint32_t e = group_entry(a, g, key, len);
+          bool mine = false;  // a claim posts the claimant's own number
+          const uint32_t e = group_entry(a, g, key, len, &mine);
           if (e == 0xFFFFFFFFu) {
             atomicCAS(&a.ctl->err, 0, (int)GLEAM_ERR_INTERNAL);
             ch.ent[g] = 0xFFFFFFFFu;
@@ -988,7 +1005,7 @@ __device__ __forceinline__ void resolve_rank(const DedupArgs& a, uint32_t G, uin
           } else {
             ch.ent[g] = e;
             ch.res[g] = kResUnresolved;
-            post = e;
+            if (!mine) post = e;
           }
         }
       }
@@ -1015,7 +1032,8 @@ __device__ __forceinline__ void resolve_rank(const DedupArgs& a, uint32_t G, uin
       const uint32_t g = base + lane;
       bool need = false, lead = false;
       uint32_t m = 0;
-      if (lane < W && g < N && ldcg_u32(&ch.res[g]) == kResUnresolved) {
+      const uint32_t res0 = lane < W && g < N ? ldcg_u32(&ch.res[g]) : kResHit0;
+      if (res0 == kResUnresolved) {
         m = ~ldcg_u32(&a.tbl[ch.ent[g]].minv);
         if (m == g) {
           ch.res[g] = kResLeader | round;
@@ -1031,6 +1049,17 @@ __device__ __forceinline__ void resolve_rank(const DedupArgs& a, uint32_t G, uin
           stay = true;
         } else {
           need = true;
+        }
+      }
+      if (counted) {
+        // (phase A made leaders of the chunks that are never cached)
+        const bool first = round == 1 && (res0 & kResLeader);
+        const unsigned mb = __ballot_sync(0xffffffffu, lead || first);
+        const unsigned sb = __ballot_sync(0xffffffffu, lead || (first && !(res0 & kResNoSlot)));
+        if (lane == 0 && mb) {
+          const uint32_t range = base / (uint32_t)per;
+          atomicAdd(&a.bcount[range], (uint32_t)__popc(mb));
+          if (sb) atomicAdd(&a.bcount[G + range], (uint32_t)__popc(sb));
         }
       }
       if (a.classes) {
@@ -1139,37 +1168,35 @@ __device__ __forceinline__ void resolve_rank(const DedupArgs& a, uint32_t G, uin
     ++round;
   }
 
+  // A verify reject: the cache had a key+length candidate, or an earlier miss of
+  // the call has this key and length (another leader of a later round; with
+  // classes, an earlier leader of the class).  And the miss's entry of the group
+  // table is left zeroed for the next call: every claimed entry belongs to a
+  // group with at least one leader.
+  auto settle_leader = [&](uint32_t g, uint32_t r) {
+    bool earlier;
+    if (a.classes) {
+      const uint32_t cl = (uint32_t)ch.cls[g];  // in range unless the call failed
+      earlier = cl <= a.tbl_mask && ~ldcg_u32(&a.cls_tbl[cl].minv) < g;
+    } else {
+      earlier = (r & kResRoundMask) > 1;
+    }
+    const bool rej = !(r & kResNoSlot) && (ch.status[g] == kMissCand || earlier);
+    if (rej) ch.res[g] = r | kResReject;
+    const uint32_t e = ch.ent[g];
+    if (e != 0xFFFFFFFFu) a.tbl[e] = CallEntry{0u, 0u};
+  };
+
   // ---- D1: misses per contiguous block range --------------------------------
-  const uint64_t per = (((uint64_t)N + G - 1) / G + 31) & ~31ull;
-  const uint32_t lo = (uint32_t)min((uint64_t)N, bid * per);
-  const uint32_t hi = (uint32_t)min((uint64_t)N, lo + per);
   unsigned long long before = 0, total = 0, sbefore = 0, stotal = 0, evict = 0;
-  if (ok) {
+  if (ok && !counted) {
     uint32_t cnt = 0, scnt = 0;
     for (uint32_t g = lo + threadIdx.x; g < hi; g += kThreads) {
       const uint32_t r = ldcg_u32(&ch.res[g]);
       if (r & kResLeader) {
         ++cnt;
         if (!(r & kResNoSlot)) ++scnt;
-        // a verify reject: the cache had a key+length candidate, or an
-        // earlier miss of the call has this key and length (another leader
-        // of a later round; with classes, an earlier leader of the class)
-        bool earlier;
-        if (a.classes) {
-          const uint32_t cl = (uint32_t)ch.cls[g];  // in range unless the call failed
-          earlier = cl <= a.tbl_mask && ~ldcg_u32(&a.cls_tbl[cl].minv) < g;
-        } else {
-          earlier = (r & kResRoundMask) > 1;
-        }
-        const bool rej = !(r & kResNoSlot) && (ch.status[g] == kMissCand || earlier);
-        if (rej) ch.res[g] = r | kResReject;
-        // leave the group table zeroed for the next call: every claimed entry
-        // belongs to a group with at least one leader
-        const uint32_t e = ch.ent[g];
-        if (e != 0xFFFFFFFFu) {
-          a.tbl[e].owner = 0u;
-          a.tbl[e].minv = 0u;
-        }
+        settle_leader(g, r);
       }
     }
     const unsigned long long c = block_sum<unsigned long long>(cnt, red64);
@@ -1231,6 +1258,7 @@ __device__ __forceinline__ void resolve_rank(const DedupArgs& a, uint32_t G, uin
       const uint32_t rv = valid ? ldcg_u32(&ch.res[g]) : 0u;
       const bool miss = valid && (rv & kResLeader);
       const bool stored = miss && !(rv & kResNoSlot);
+      if (counted && miss) settle_leader(g, rv);
       const uint32_t mb = __ballot_sync(0xffffffffu, miss);
       const uint32_t sb = __ballot_sync(0xffffffffu, stored);
       if (lane == 0) {
@@ -1263,7 +1291,9 @@ __device__ __forceinline__ void resolve_rank(const DedupArgs& a, uint32_t G, uin
       srunning += swarp_cnt[0];
       __syncthreads();
     }
-    ok = grid_barrier(a.ctl, G, a.wait_ns, false);
+    // no barrier: what reads the ranks follows a kernel boundary or a barrier
+    // of its own, and an eviction's first barrier comes before it writes
+    // anything that a slower block may still read here
   }
   if (ok && evict && G == 1) {  // its barriers did not read the error word
     if (threadIdx.x == 0) s_err1 = ld_volatile_s32(&a.ctl->err);
