@@ -66,7 +66,8 @@ enum StatIdx {
   ST_REJECTS, ST_SLOTS_USED, ST_BYTES_USED, ST_EVICTIONS, ST_SPEC_CHUNKS, ST_COUNT
 };
 
-// Per-call control block; starts zeroed and every dedup kernel leaves it zeroed.
+// Per-call control block; starts zeroed and every dedup kernel leaves it zeroed
+// (but for `published`).
 struct DevCtl {
   unsigned int bar_count;  // grid-barrier arrivals of the call (nblocks per barrier)
   unsigned int copy_next;  // next piece to hand out (one-launch resolve + pack copies)
@@ -92,6 +93,10 @@ struct DevCtl {
   // write-through of likely misses (HashArgs::spec_mode)
   unsigned long long spec_tried;        // chunks the hash kernel wrote ahead
   unsigned long long spec_used;         // misses whose copies that made unnecessary
+  // Away from bar_count, which every block polls: next to it, the blocks' stores
+  // of any_miss before they arrive at the barrier made k_dedup 10% slower.
+  unsigned int any_miss;   // k_dedup found a chunk that is not a cache hit
+  unsigned int published;  // DedupArgs::seq of the last call that k_dedup published itself
 };
 
 // Position of a key in a power-of-two table: the 64-bit finaliser of
@@ -261,6 +266,7 @@ struct DedupArgs {
   uint32_t* spec_mirror;
   // the hash kernel claimed the misses' groups (HashArgs::claim_tbl)
   uint32_t pre_claimed;
+  uint32_t seq;              // number of the call, never 0
   // one-launch resolve + pack: pieces of misses a warp takes at a time from a
   // counter of the call (1..32), or 0 for an equal share per warp
   uint32_t copy_grab;
@@ -425,11 +431,17 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 // one to wait for: the block barrier orders its memory accesses, and it
 // returns !skip without reading the error word (a caller about to make a
 // change that an error must prevent reads it itself).
+// any_miss, if given, receives whether DevCtl::any_miss was set by then (read
+// by one thread together with the error word).
 __device__ __forceinline__ bool grid_barrier(DevCtl* ctl, unsigned int nblocks,
-                                             unsigned long long wait_ns, bool skip) {
+                                             unsigned long long wait_ns, bool skip,
+                                             bool* any_miss = nullptr) {
   __shared__ int s_ok;  // the block's verdict, so that every thread agrees
   __syncthreads();
-  if (nblocks == 1) return !skip;
+  if (nblocks == 1) {
+    if (any_miss) *any_miss = *reinterpret_cast<const volatile unsigned int*>(&ctl->any_miss) != 0;
+    return !skip;
+  }
   if (threadIdx.x == 0 && !skip) {
     // arrivals only grow during a call: this barrier is passed once the
     // count reaches the next multiple of nblocks (no reset, no second flag)
@@ -449,9 +461,15 @@ __device__ __forceinline__ bool grid_barrier(DevCtl* ctl, unsigned int nblocks,
     }
     __threadfence();
   }
-  if (threadIdx.x == 0) s_ok = (!skip && ld_volatile_s32(&ctl->err) == 0) ? 1 : 0;
+  if (threadIdx.x == 0) {
+    const unsigned int any =
+        any_miss ? *reinterpret_cast<const volatile unsigned int*>(&ctl->any_miss) : 0u;
+    s_ok = ((!skip && ld_volatile_s32(&ctl->err) == 0) ? 1 : 0) | (any ? 2 : 0);
+  }
   __syncthreads();
-  return s_ok != 0;
+  const int v = s_ok;
+  if (any_miss) *any_miss = (v & 2) != 0;
+  return (v & 1) != 0;
 }
 
 // Payload owning global chunk g: the last p with chunk_base <= g (empty
