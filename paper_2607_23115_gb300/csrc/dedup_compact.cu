@@ -38,6 +38,7 @@
 // grid of one block (every grid barrier a block barrier), so that the call
 // costs one launch and no kernel boundary.
 #include <algorithm>
+#include <atomic>
 
 #include "gleam_internal.cuh"
 #include "staged_hash.cuh"
@@ -2738,33 +2739,37 @@ int dedup_chunks_per_block() { return GLEAM_DEDUP_CHUNKS_PER_BLOCK; }
 // copies' buffers.
 constexpr uint32_t pack_smem_bytes(bool plain) { return plain ? 0u : kPackSmem; }
 
-template <typename K>
-int blocks_per_sm(K kern, uint32_t smem) {
-  int nb = 0;
-  if (cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
+// Co-resident blocks per SM of a kernel (0: unknown), asked for once (the
+// pool's GPUs are all alike): a query costs tens of microseconds of every cache
+// creation.
+template <auto kKern>
+int blocks_per_sm(uint32_t smem) {
+  static std::atomic<int> known{0};
+  int nb = known.load();
+  if (nb > 0) return nb;
+  if (cudaFuncSetAttribute((const void*)kKern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
           cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, kThreads, smem) != cudaSuccess)
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kKern, kThreads, smem) != cudaSuccess)
     return 0;
+  known.store(nb);
   return nb;
 }
 
 // Co-resident blocks per SM of the pack kernel.
-int pack_blocks_per_sm() { return blocks_per_sm(k_pack<false>, pack_smem_bytes(false)); }
+int pack_blocks_per_sm() { return blocks_per_sm<k_pack<false>>(pack_smem_bytes(false)); }
 
 // Co-resident blocks per SM of the one-launch resolve + pack kernel (its grid
 // barriers need every block of the grid resident at once).
 int resolve_pack_blocks_per_sm() {
-  return std::min({blocks_per_sm(k_resolve_pack<false>, pack_smem_bytes(false)),
-                   blocks_per_sm(k_resolve_pack<true>, pack_smem_bytes(true)),
-                   blocks_per_sm(k_resolve_direct<false>, pack_smem_bytes(false)),
-                   blocks_per_sm(k_resolve_direct<true>, pack_smem_bytes(true))});
+  return std::min({blocks_per_sm<k_resolve_pack<false>>(pack_smem_bytes(false)),
+                   blocks_per_sm<k_resolve_pack<true>>(pack_smem_bytes(true)),
+                   blocks_per_sm<k_resolve_direct<false>>(pack_smem_bytes(false)),
+                   blocks_per_sm<k_resolve_direct<true>>(pack_smem_bytes(true))});
 }
 
 // Co-resident blocks per SM for the cooperative launch (capped).
 int dedup_blocks_per_sm() {
-  int nb = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_dedup, kThreads, 0) != cudaSuccess)
-    return 0;
+  const int nb = blocks_per_sm<k_dedup>(0);
   return nb < GLEAM_DEDUP_BLOCKS_PER_SM ? nb : GLEAM_DEDUP_BLOCKS_PER_SM;
 }
 

@@ -74,6 +74,7 @@ struct gleam_cache {
   // and an upper bound of the slots in use (no device read needed), which
   // tells when a call of an LRU cache cannot need an eviction
   uint64_t small_max_chunks = 0;
+  bool small_forced = false;  // set by GLEAM_DEBUG_SMALL_CALLS: whatever their hash
   uint64_t slots_bound = 0;
 
   // write-through of likely misses (HashArgs::spec_mode)
@@ -758,7 +759,6 @@ int enqueue(gleam_cache* c, const gleam_payload_t* payloads, uint64_t count,
     grid = std::max(grid, std::min(2, c->coop_max_blocks));  // someone must be left waiting
     if (d.skip_block >= grid) d.skip_block = grid - 1;
   }
-  const bool fused = small_call(c, Ntot, nbytes, d.skip_block);
   const bool chain = chain_call(c, Ntot, nbytes, d.skip_block);
   // a larger call on its own chains its launches too, on its full grids
   const bool pdl = chain || (d.skip_block < 0 && !(c->flags & GLEAM_OVERLAP_CALLS));
@@ -768,12 +768,24 @@ int enqueue(gleam_cache* c, const gleam_payload_t* payloads, uint64_t count,
   h.wait_late = chain && (c->flags & GLEAM_OVERLAP_CALLS) &&
                         !(c->flags & (GLEAM_PAPER_IDS | GLEAM_EVICT_LRU))
                     ? 1u : 0u;
+  // A call hashed with a warp per chunk is faster as chained launches than as
+  // one block, whose few warps run the chunks' chains among all else.  One
+  // payload, two launches against one block: one chunk of 64 KiB 45 us against
+  // 93, of 16 KiB 21 against 31, of 4 KiB 13.4 against 14.8, 64 chunks of 4 KiB
+  // 20 against 32; batches, three launches: 4 payloads of one 64 KiB chunk 66
+  // against 117, 60 of one 4 KiB chunk 40 against 51.  (Chunks of 1 KiB keep the
+  // one block: 11.5 us against 12.5 for one, and where calls overlap chunks
+  // under 32 KiB, 5.4 against 6.7, and batches.)
+  const bool direct = chain && count == 1 && !d.classes && !d.lru;
+  const bool fused =
+      small_call(c, Ntot, nbytes, d.skip_block) &&
+      (c->small_forced || !hash_is_lone(h) || !(direct || !(c->flags & GLEAM_OVERLAP_CALLS)));
   // host payloads too: a chunk written ahead then spares the pack a second
   // read over the CPU-GPU link (managed memory stays out)
   set_spec(c, &h, &d, aligned && packed_aligned && !chk.saw_managed() && !h.wait_late);
   // a payload resolved by the one-launch kernel: its staged hash kernel
   // claims the misses' groups as it records them
-  const bool one_launch = !fused && chain && count == 1 && !d.classes && !d.lru;
+  const bool one_launch = !fused && direct;
   int rp_grid = 1;
   if (one_launch) {
     // at most one chunk per thread, and one block per kChainBytesPerBlock of
@@ -1254,6 +1266,7 @@ int gleam_cache_debug_set(gleam_cache_t* c, int what, int64_t value) {
   if (what == GLEAM_DEBUG_SMALL_CALLS) {
     if (value < 0 || value > (int64_t)kMaxChunks) return GLEAM_ERR_INVALID_ARG;
     c->small_max_chunks = (uint64_t)value;
+    c->small_forced = true;
     return GLEAM_OK;
   }
   if (what == GLEAM_DEBUG_CLOCK) {

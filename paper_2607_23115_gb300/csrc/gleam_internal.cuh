@@ -285,6 +285,8 @@ cudaError_t launch_hash(const HashArgs& a, bool aligned, cudaStream_t s, bool pd
 // Whether launch_hash runs the staged XXH64 kernel for these arguments (the
 // one that can claim groups, HashArgs::claim_tbl).
 bool hash_is_staged(const HashArgs& a);
+// Whether it runs the one with a warp per chunk.
+bool hash_is_lone(const HashArgs& a);
 // Loads the hash kernels' device code on the current GPU (cache creation does
 // it, so that no later call loads code, which allocates device memory).
 cudaError_t load_hash_kernels();

@@ -475,6 +475,10 @@ cudaError_t load_hash_kernels() {
   return cudaFuncGetAttributes(&fa, k_hash_probe_staged<true, false, true>);
 }
 
+bool hash_is_lone(const HashArgs& a) {
+  return a.Ntot > 0 && !(a.index != nullptr && a.paper) && lone_call(a);
+}
+
 bool hash_is_staged(const HashArgs& a) { return a.Ntot > 0 && !(a.index != nullptr && a.paper); }
 
 cudaError_t launch_hash(const HashArgs& a, bool aligned, cudaStream_t s, bool pdl) {

@@ -88,3 +88,22 @@ def test_batch_of_mixed_payloads():
             parts[2] = parts[2].clone()
             parts[2][::3 * C] ^= 1
         compare_cache(gc, oc, check_bytes=200)
+
+
+def test_small_calls_either_way():
+    """Calls of at most 64 chunks as the library runs them, and with the
+    single-block kernel asked for: equal to the oracle both times."""
+    C = 4 * KiB
+    for limit in (None, 64):
+        gc, oc = Cache(600 * C, C), oracle.OracleCache(600 * C, C)
+        with gc:
+            if limit is not None:
+                gc.debug_set(B.GLEAM_DEBUG_SMALL_CALLS, limit)
+            for n in (1, 100, 511, 512, C - 1, C, C + 1, 9 * C + 700, 63 * C, 64 * C - 5):
+                host = W.random_bytes(n, seed=n)
+                for offset in (0, 8, 0):
+                    dedup_both(gc, oc, host, offset=offset)
+                host = host.clone()
+                host[n // 2] ^= 16
+                dedup_both(gc, oc, host)
+            compare_cache(gc, oc, check_bytes=300)
