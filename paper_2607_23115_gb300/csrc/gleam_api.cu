@@ -560,13 +560,15 @@ constexpr uint64_t kChainDedupBytes = 2ull << 20;
 constexpr uint64_t kChainSmallCall = 4ull << 20;
 constexpr uint64_t kChainBytesPerBlock = GLEAM_CHAIN_BYTES_PER_BLOCK;
 // Without GLEAM_OVERLAP_CALLS a call overlaps the next only by the launch, so
-// its one-launch resolve kernel may take a block per 512 KiB, up to one per SM
-// (a 64 MiB call of 16,384 chunks: 0.101 -> 0.092 ms); with it, blocks that
-// wait for an earlier call hold resources that the calls in flight want.
-#ifndef GLEAM_SOLO_KIB_PER_BLOCK
-#define GLEAM_SOLO_KIB_PER_BLOCK 512
-#endif
-constexpr uint64_t kSoloBytesPerBlock = (uint64_t)GLEAM_SOLO_KIB_PER_BLOCK << 10;
+// its one-launch resolve kernel may take a block per kSoloBytesPerBlock, up to
+// all that are resident at once (a 64 MiB call of 16,384 chunks, half of them
+// misses: 81 us with a block per 512 KiB and at most one per SM, 72 with one
+// per 256 KiB, 71 with 128 or 64 KiB; a Llama-3-8B layer, one call per tensor
+// 514 / 505 / 500 / 499), and calls under kSoloSmallCall one per 512 KiB; with
+// it, blocks that wait for an earlier call hold resources that the calls in
+// flight want.
+constexpr uint64_t kSoloSmallCall = 1ull << 20, kSmallBytesPerBlock = 512ull << 10;
+constexpr uint64_t kSoloBytesPerBlock = 64ull << 10;
 #ifndef GLEAM_OVERLAP_COPY_GRAB
 #define GLEAM_OVERLAP_COPY_GRAB 8
 #endif
@@ -791,12 +793,10 @@ int enqueue(gleam_cache* c, const gleam_payload_t* payloads, uint64_t count,
     // at most one chunk per thread, and one block per kChainBytesPerBlock of
     // payload so that the misses' copies spread
     const bool solo = !(c->flags & GLEAM_OVERLAP_CALLS);
-    const uint64_t per_block =
-        solo || nbytes < kChainSmallCall ? kSoloBytesPerBlock : kChainBytesPerBlock;
-    const uint64_t cap =
-        solo ? (uint64_t)std::min(c->rp_max_blocks,
-                                  std::max(kChainPackBlocks, one_per_sm(c)))
-             : (uint64_t)kChainPackBlocks;
+    const uint64_t per_block = nbytes < (solo ? kSoloSmallCall : kChainSmallCall)
+                                   ? kSmallBytesPerBlock
+                               : solo ? kSoloBytesPerBlock : kChainBytesPerBlock;
+    const uint64_t cap = (uint64_t)(solo ? c->rp_max_blocks : kChainPackBlocks);
     const uint64_t want = std::max<uint64_t>((Ntot + dedup_threads() - 1) / dedup_threads(),
                                              (nbytes + per_block - 1) / per_block);
     rp_grid = (int)std::min<uint64_t>(std::max<uint64_t>(1, want), cap);
