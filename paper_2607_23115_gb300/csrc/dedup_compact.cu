@@ -1261,6 +1261,7 @@ __device__ __forceinline__ bool resolve_rank(const DedupArgs& a, uint32_t G, uin
   }
   if (ok) {
     unsigned long long running = before, srunning = sbefore;
+    uint32_t n_ahead = 0;  // misses that the hash kernel wrote where they belong
     for (uint32_t t = lo; t < hi; t += kThreads) {
       const uint32_t g = t + threadIdx.x;
       const bool valid = g < hi;
@@ -1292,13 +1293,21 @@ __device__ __forceinline__ bool resolve_rank(const DedupArgs& a, uint32_t G, uin
         const uint32_t r = (uint32_t)(running + warp_off[w] + __popc(mb & below));
         ch.rank[g] = r;
         if (miss) ch.order[r] = g;
-        if (stored) ch.srank[g] = (uint32_t)(srunning + swarp_off[w] + __popc(sb & below));
+        if (stored) {
+          const uint32_t sr = (uint32_t)(srunning + swarp_off[w] + __popc(sb & below));
+          ch.srank[g] = sr;
+          n_ahead += a.spec_active && evict == 0 && sr == g && ch.spec[g];
+        }
         const uint32_t p = ch.pidx[g];
         if (g == desc(a, p).chunk_base) a.pstart[p] = r;
       }
       running += warp_cnt[0];
       srunning += swarp_cnt[0];
       __syncthreads();
+    }
+    if (a.spec_active) {
+      const unsigned long long s = block_sum<unsigned long long>(n_ahead, red64);
+      if (threadIdx.x == 0 && s) atomicAdd(&a.ctl->spec_ahead, s);
     }
     // no barrier: what reads the ranks follows a kernel boundary or a barrier
     // of its own, and an eviction's first barrier comes before it writes
@@ -1439,7 +1448,7 @@ __device__ __forceinline__ void finish_call(const DedupArgs& a, uint32_t G,
     c->acc_stored = c->acc_stored_bytes = 0;
     c->acc_distinct = c->evict_k = c->lru_below = c->lru_ties = c->acc_victim_bytes = 0;
     c->lru_hi = c->lru_cut = 0;
-    c->spec_tried = c->spec_used = 0;
+    c->spec_tried = c->spec_used = c->spec_ahead = 0;
     c->done = 0;
   }
   __threadfence();
@@ -1511,7 +1520,7 @@ __device__ __forceinline__ void pack_publish(const DedupArgs& a, uint32_t G, uin
   __shared__ unsigned long long red64[kWarps];
   __shared__ unsigned long long s_slots0, s_total, s_evict;
   // a grid of one block keeps its totals here instead of in the control block
-  __shared__ unsigned long long s_stored, s_vbytes, s_sum[7];
+  __shared__ unsigned long long s_stored, s_vbytes, s_ahead, s_sum[7];
   __shared__ int s_err;
   const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const uint32_t N = (uint32_t)a.Ntot;
@@ -1523,6 +1532,7 @@ __device__ __forceinline__ void pack_publish(const DedupArgs& a, uint32_t G, uin
     s_evict = __ldcg(&a.ctl->evict_k);
     s_stored = __ldcg(&a.ctl->acc_stored);
     s_vbytes = __ldcg(&a.ctl->acc_victim_bytes);
+    s_ahead = a.spec_active ? __ldcg(&a.ctl->spec_ahead) : 0ull;
     for (int k = 0; k < 7; ++k) s_sum[k] = 0;
   }
   __syncthreads();
@@ -1675,21 +1685,27 @@ __device__ __forceinline__ void pack_publish(const DedupArgs& a, uint32_t G, uin
     auto written_ahead = [&](uint32_t gg, uint32_t sr) {
       return a.spec_active && evict == 0 && sr == gg && ch.spec[gg];
     };
-    // Without the write-through the warps take their steps from a counter of
+    // Mostly the warps take their steps from a counter of
     // the call instead (each asks for its next step before it copies the
     // current one), so that warps on SMs that copy faster take more: steps of
     // 32 pieces, then, from kFinePerWarp pieces per warp before the end,
     // steps of kFineStep, so that the last steps end together.
-    // The static ranges remain where the hash kernel wrote likely misses ahead
-    // (the steps then copy little, and the counter's round trip would be most
-    // of a step) and for counts the 32-bit counter cannot hold.
-    const bool grab = !a.spec_active && npieces < (1ull << 31);
+    // The static ranges remain where the hash kernel wrote at least half of the
+    // misses ahead (the steps then copy little, and the counter's round trip
+    // would be most of a step), where a warp has less than a fine step (a batch
+    // of 665 misses of 64 KiB, 5.8 pieces a warp: 246 us so, 252 with the
+    // counter), and for counts the 32-bit counter cannot hold.
+    // Where it wrote all of them ahead (a first load) there is nothing to copy,
+    // and no step looks its pieces up to find that out (498 MB in 148 payloads,
+    // none cached: 344 -> 341 us).
+    const bool grab =
+        2 * s_ahead < total && npieces >= kFineStep * nw && npieces < (1ull << 31);
     const unsigned long long coarse =
         npieces > nw * kFinePerWarp ? (npieces - nw * kFinePerWarp) / 32 : 0ull;
     auto step_at = [&](unsigned long long v) {  // first piece of the counter's v-th step
       return v <= coarse ? 32 * v : 32 * coarse + kFineStep * (v - coarse);
     };
-    unsigned long long step = plo, step_end = phi;
+    unsigned long long step = plo, step_end = s_ahead == total ? plo : phi;
     if (grab) {
       uint32_t b0 = 0;
       if (lane == 0) b0 = atomicAdd(&a.ctl->copy_next, 1u);

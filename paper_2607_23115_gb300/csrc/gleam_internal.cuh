@@ -93,6 +93,7 @@ struct DevCtl {
   // write-through of likely misses (HashArgs::spec_mode)
   unsigned long long spec_tried;        // chunks the hash kernel wrote ahead
   unsigned long long spec_used;         // misses whose copies that made unnecessary
+  unsigned long long spec_ahead;        // those, as the resolve kernel knows them before the pack
   // Away from bar_count, which every block polls: next to it, the blocks' stores
   // of any_miss before they arrive at the barrier made k_dedup 10% slower.
   unsigned int any_miss;   // k_dedup found a chunk that is not a cache hit
