@@ -551,14 +551,13 @@ constexpr int kChainPackBlocks = GLEAM_CHAIN_PACK_BLOCKS;
 constexpr uint64_t kChainDedupBytes = 2ull << 20;
 // Overlapping calls: a block of the one-launch kernel per 2 MiB of payload
 // (Llama-3-8B, one call per tensor: 1,558-1,571 GB/s, against 1,480-1,495
-// with 1 MiB), or per 512 KiB for calls under 4 MiB, whose copies would
-// otherwise fall to one block (the 10,000-call stream's calls of 256 KiB-
-// 1 MiB: 38.8 -> 34.2 us each).
-#ifndef GLEAM_CHAIN_BYTES_PER_BLOCK
-#define GLEAM_CHAIN_BYTES_PER_BLOCK (2ull << 20)
-#endif
-constexpr uint64_t kChainSmallCall = 4ull << 20;
-constexpr uint64_t kChainBytesPerBlock = GLEAM_CHAIN_BYTES_PER_BLOCK;
+// with 1 MiB), but for calls that are mostly misses, whose copies would else
+// fall to few blocks, one per 256 KiB up to kOverlapBlocks (first loads of
+// 16-KiB chunks, one call of 300 / 1,200 of them: 98 / 116 us with one per 2 MiB,
+// 55 / 116 with at least 8, 41 / 85 with 16, 34 / 59 with 32; but a Llama-3-8B
+// layer, a tenth of it changed, 317 / 319 / 317 / 324).
+constexpr uint64_t kChainBytesPerBlock = 2ull << 20;
+constexpr uint64_t kOverlapFewBytes = 256ull << 10, kOverlapBlocks = 16;
 // Without GLEAM_OVERLAP_CALLS a call overlaps the next only by the launch, so
 // its one-launch resolve kernel may take a block per kSoloBytesPerBlock, up to
 // all that are resident at once (a 64 MiB call of 16,384 chunks, half of them
@@ -790,15 +789,17 @@ int enqueue(gleam_cache* c, const gleam_payload_t* payloads, uint64_t count,
   const bool one_launch = !fused && direct;
   int rp_grid = 1;
   if (one_launch) {
-    // at most one chunk per thread, and one block per kChainBytesPerBlock of
-    // payload so that the misses' copies spread
+    // at most one chunk per thread, and more blocks by the payload's bytes, so
+    // that the misses' copies spread
     const bool solo = !(c->flags & GLEAM_OVERLAP_CALLS);
-    const uint64_t per_block = nbytes < (solo ? kSoloSmallCall : kChainSmallCall)
-                                   ? kSmallBytesPerBlock
-                               : solo ? kSoloBytesPerBlock : kChainBytesPerBlock;
+    auto blocks_of = [&](uint64_t bytes) { return (nbytes + bytes - 1) / bytes; };
+    const uint64_t copy_blocks =
+        solo ? blocks_of(nbytes < kSoloSmallCall ? kSmallBytesPerBlock : kSoloBytesPerBlock)
+             : std::max(std::min(blocks_of(kOverlapFewBytes), kOverlapBlocks),
+                        blocks_of(kChainBytesPerBlock));
     const uint64_t cap = (uint64_t)(solo ? c->rp_max_blocks : kChainPackBlocks);
     const uint64_t want = std::max<uint64_t>((Ntot + dedup_threads() - 1) / dedup_threads(),
-                                             (nbytes + per_block - 1) / per_block);
+                                             copy_blocks);
     rp_grid = (int)std::min<uint64_t>(std::max<uint64_t>(1, want), cap);
   }
   // overlapping calls give the one-launch kernel few blocks (a block per
