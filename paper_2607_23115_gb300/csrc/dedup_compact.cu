@@ -2332,15 +2332,24 @@ __device__ __forceinline__ void resolve_direct(const DedupArgs& a, uint32_t G, u
   const bool miss = valid && (sh.bits[g >> 5] >> (g & 31) & 1u);
 
   if (sh.shared) {
-    // a group may be shared: the general algorithm, from cleared outputs
-    for (uint32_t k = bid * kThreads + threadIdx.x; k < nw; k += G * kThreads) P.mask[k] = 0;
+    // a group may be shared: the general algorithm, from cleared outputs, on the
+    // first Gg blocks, each with a larger share of the chunks
+    const uint32_t Gg = min(G, a.general_blocks);
+    if (bid >= Gg) return;
+    const uint32_t pg = (N + Gg - 1) / Gg;  // <= kThreads, too
+    const uint32_t c = bid * pg + threadIdx.x;
+    const bool mine = threadIdx.x < pg && c < N;
+    if (pg > kThreads && threadIdx.x == 0) atomicCAS(&a.ctl->err, 0, (int)GLEAM_ERR_INTERNAL);
+    for (uint32_t k = bid * kThreads + threadIdx.x; k < nw; k += Gg * kThreads) P.mask[k] = 0;
     if (bid == 0 && threadIdx.x == 0 && P.result) {
       gleam_result_t* r = P.result;
       r->n_miss = r->n_hit_cache = r->n_hit_intra = r->verify_rejects = r->miss_bytes = 0;
     }
-    if (valid && !miss) ch.res[g] = kResHit0;
-    const uint32_t len = valid ? ch.len[g] : 0u;
-    resolve_pack_general<kPlain>(a, G, bid, smem, ok, true, miss, e, key, len, g);
+    const bool grouped = mine && (sh.bits[c >> 5] >> (c & 31) & 1u);
+    if (mine && !grouped) ch.res[c] = kResHit0;
+    resolve_pack_general<kPlain>(a, Gg, bid, smem, ok, true, grouped,
+                                 grouped ? ch.ent[c] : 0xFFFFFFFFu, grouped ? ch.key[c] : 0ull,
+                                 grouped ? ch.len[c] : 0u, c);
     return;
   }
 
@@ -2791,6 +2800,10 @@ int dedup_blocks_per_sm() {
 
 cudaError_t launch_dedup(const DedupArgs& a, int grid, int pack_grid, cudaStream_t s, bool pdl) {
   cudaError_t e;
+  // chained, and so small that several caches' calls are resident together:
+  // a regular launch, which may start early; else a cooperative one, which
+  // starts once all of its blocks fit beside whatever else is running
+  pdl = pdl && grid <= kRegularDedupBlocks;
   if (pdl) {
     e = launch_kernel(k_dedup, dim3(grid), dim3(kThreads), 0, s, true, a);
   } else {

@@ -797,7 +797,12 @@ int enqueue(gleam_cache* c, const gleam_payload_t* payloads, uint64_t count,
         solo ? blocks_of(nbytes < kSoloSmallCall ? kSmallBytesPerBlock : kSoloBytesPerBlock)
              : std::max(std::min(blocks_of(kOverlapFewBytes), kOverlapBlocks),
                         blocks_of(kChainBytesPerBlock));
-    const uint64_t cap = (uint64_t)(solo ? c->rp_max_blocks : kChainPackBlocks);
+    // grid barriers (always without the hash kernel's claims, else where a group
+    // is shared) want no more than a block per SM, so that two caches' calls fit
+    const int barrier_blocks = std::min(c->rp_max_blocks, std::max(kChainPackBlocks, one_per_sm(c)));
+    d.general_blocks = (uint32_t)barrier_blocks;
+    const uint64_t cap = (uint64_t)(!solo ? kChainPackBlocks
+                                    : hash_is_staged(h) ? c->rp_max_blocks : barrier_blocks);
     const uint64_t want = std::max<uint64_t>((Ntot + dedup_threads() - 1) / dedup_threads(),
                                              copy_blocks);
     rp_grid = (int)std::min<uint64_t>(std::max<uint64_t>(1, want), cap);

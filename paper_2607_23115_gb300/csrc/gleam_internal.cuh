@@ -268,6 +268,10 @@ struct DedupArgs {
   // the hash kernel claimed the misses' groups (HashArgs::claim_tbl)
   uint32_t pre_claimed;
   uint32_t seq;              // number of the call, never 0
+  // k_resolve_direct: blocks that run the general algorithm, with its grid
+  // barriers, where a group is shared (the others leave): few enough that the
+  // calls of two caches fit the GPU together
+  uint32_t general_blocks;
   // one-launch resolve + pack: pieces of misses a warp takes at a time from a
   // counter of the call (1..32), or 0 for an equal share per warp
   uint32_t copy_grab;
@@ -291,12 +295,14 @@ bool hash_is_lone(const HashArgs& a);
 // Loads the hash kernels' device code on the current GPU (cache creation does
 // it, so that no later call loads code, which allocates device memory).
 cudaError_t load_hash_kernels();
-// The cooperative resolve/rank kernel on `grid` blocks, then the pack kernel
-// (masks, indices, copies, inserts, publish) on `pack_grid` blocks.  pdl: both
-// launched with programmatic stream serialization, the resolve kernel then as
-// a regular launch (a cooperative one is never launched early); its grid must
-// fit the GPU at once, and every block of it is resident before anything
-// later on the stream can start, so its grid barriers still complete.
+// The resolve/rank kernel on `grid` blocks, then the pack kernel (masks, indices,
+// copies, inserts, publish) on `pack_grid` blocks.  pdl: both launched with
+// programmatic stream serialization if the grid is at most kRegularDedupBlocks,
+// the resolve kernel then as a regular launch (a cooperative one is never
+// launched early): every block of it is resident before anything later on the
+// stream can start, and several caches' calls fit the GPU at once, so its grid
+// barriers still complete.  Else the resolve kernel is a cooperative launch.
+constexpr int kRegularDedupBlocks = 32;
 cudaError_t launch_dedup(const DedupArgs& a, int grid, int pack_grid, cudaStream_t s,
                          bool pdl = false);
 // Resolve, rank, pack and publish of a one-payload call in one launch on
