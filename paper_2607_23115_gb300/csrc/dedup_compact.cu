@@ -936,6 +936,10 @@ __device__ __forceinline__ bool resolve_rank(const DedupArgs& a, uint32_t G, uin
   __shared__ unsigned long long s_slots0;
   __shared__ unsigned long long sred[kThreads];
   __shared__ int s_err1, s_any;  // s_any: a chunk of the block's is not a cache hit
+  // chunks of a block's contiguous range; here, and the range's bounds taken after
+  // the rounds, so that the compares' loads find registers (1 GiB of 64 KiB
+  // chunks, half of them copies: 201 us the kernel, 286 with the bounds live)
+  __shared__ uint32_t s_per;
 
   const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const uint32_t tid = bid * kThreads + threadIdx.x;
@@ -948,10 +952,6 @@ __device__ __forceinline__ bool resolve_rank(const DedupArgs& a, uint32_t G, uin
   const unsigned long long my_slots0 =
       threadIdx.x == 0 ? *(volatile const unsigned long long*)&a.dstats[ST_SLOTS_USED] : 0ull;
 
-  // contiguous chunk range of each block, for the ranks
-  const uint64_t per = (((uint64_t)N + G - 1) / G + 31) & ~31ull;
-  const uint32_t lo = (uint32_t)min((uint64_t)N, bid * per);
-  const uint32_t hi = (uint32_t)min((uint64_t)N, lo + per);
   // the rounds count the misses of every range as they find them (a warp step's
   // 32 chunks lie in one range), so that the ranks need no counting pass and no
   // barrier after it; a grid of one, and KEY16 classes, whose rejects wait for
@@ -960,7 +960,10 @@ __device__ __forceinline__ bool resolve_rank(const DedupArgs& a, uint32_t G, uin
 
   // ---- A: clear outputs, round-1 claims; LRU: stamp the slots hit ----------
   if (!claimed) {
-    if (threadIdx.x == 0) s_any = 0;
+    if (threadIdx.x == 0) {
+      s_any = 0;
+      s_per = (uint32_t)((((uint64_t)N + G - 1) / G + 31) & ~31ull);
+    }
     __syncthreads();
     if (counted)
       for (uint32_t j = tid; j < 2 * G; j += nth) a.bcount[j] = 0;
@@ -1066,7 +1069,7 @@ __device__ __forceinline__ bool resolve_rank(const DedupArgs& a, uint32_t G, uin
         const unsigned mb = __ballot_sync(0xffffffffu, lead || first);
         const unsigned sb = __ballot_sync(0xffffffffu, lead || (first && !(res0 & kResNoSlot)));
         if (lane == 0 && mb) {
-          const uint32_t range = base / (uint32_t)per;
+          const uint32_t range = base / s_per;
           atomicAdd(&a.bcount[range], (uint32_t)__popc(mb));
           if (sb) atomicAdd(&a.bcount[G + range], (uint32_t)__popc(sb));
         }
@@ -1177,6 +1180,10 @@ __device__ __forceinline__ bool resolve_rank(const DedupArgs& a, uint32_t G, uin
     ++round;
   }
 
+  // contiguous chunk range of each block, for the ranks
+  const uint64_t per = (((uint64_t)N + G - 1) / G + 31) & ~31ull;
+  const uint32_t lo = (uint32_t)min((uint64_t)N, bid * per);
+  const uint32_t hi = (uint32_t)min((uint64_t)N, lo + per);
   // A verify reject: the cache had a key+length candidate, or an earlier miss of
   // the call has this key and length (another leader of a later round; with
   // classes, an earlier leader of the class).  And the miss's entry of the group
