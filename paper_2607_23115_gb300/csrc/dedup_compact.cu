@@ -1335,12 +1335,6 @@ __device__ __forceinline__ bool resolve_rank(const DedupArgs& a, uint32_t G, uin
   return false;
 }
 
-// The end of a call, run by every block: the last block to get here
-// publishes the counters and results and leaves the per-call state (group
-// table, control block) as the next call expects it.  total/stored/evict/
-// vbytes: the call's misses, stored misses, evicted slots and their bytes;
-// s_sum: a grid of one block's sums (hits, intra hits, rejects, miss bytes,
-// stored bytes, chunks written ahead, of them used), else the control block's.
 // After an error that may have stopped the leaders before they cleared their
 // entries: the whole group table (and class table), and an eviction's
 // histogram and flags.  Out of line: rare, and kept out of the code that
@@ -1357,30 +1351,43 @@ __device__ __noinline__ void clear_after_error(const DedupArgs& a) {
   }
 }
 
-__device__ __forceinline__ void finish_call(const DedupArgs& a, uint32_t G,
-                                            unsigned long long slots0,
-                                            unsigned long long total,
-                                            unsigned long long s_stored,
-                                            unsigned long long evict,
-                                            unsigned long long s_vbytes,
-                                            const unsigned long long* s_sum) {
-  const uint32_t N = (uint32_t)a.Ntot;
+// The end of a call, run by every block of its last kernel (finish_call): the
+// last block to get here publishes the counters and results and leaves the
+// per-call state (group table, control block) as the next call expects it.
+// total/stored/evict/vbytes: the call's misses, stored misses, evicted slots and
+// their bytes; s_sum: a grid of one block's sums (hits, intra hits, rejects, miss
+// bytes, stored bytes, chunks written ahead, of them used), else the control
+// block's.
+//
+// Whether the calling block is the last of n to get here; what the others wrote
+// before is then visible to it.  Called by every thread.
+__device__ __forceinline__ bool last_to_arrive(DevCtl* ctl, uint32_t n) {
   __shared__ int s_last;
   __syncthreads();
   if (threadIdx.x == 0) {
-    if (G == 1) {  // the block barrier already orders the block's own writes
+    if (n == 1) {  // the block barrier already orders the block's own writes
       s_last = 1;
     } else {
       __threadfence();
-      s_last = atomicAdd(&a.ctl->done, 1u) == G - 1;
+      s_last = atomicAdd(&ctl->done, 1u) == n - 1;
     }
   }
   __syncthreads();
-  if (!s_last) return;
-  if (G > 1) __threadfence();
+  if (!s_last) return false;
+  if (n > 1) __threadfence();
+  return true;
+}
+
+__device__ __forceinline__ void publish_call(const DedupArgs& a, bool one,
+                                             unsigned long long slots0,
+                                             unsigned long long total,
+                                             unsigned long long s_stored,
+                                             unsigned long long evict,
+                                             unsigned long long s_vbytes,
+                                             const unsigned long long* s_sum) {
+  const uint32_t N = (uint32_t)a.Ntot;
   const int err = ld_volatile_s32(&a.ctl->err);
   if (threadIdx.x == 0) {
-    const bool one = G == 1;
     const unsigned long long misses = total;
     const unsigned long long hc = one ? s_sum[0] : __ldcg(&a.ctl->acc_hits_cache);
     const unsigned long long hi2 = one ? s_sum[1] : __ldcg(&a.ctl->acc_hits_intra);
@@ -1461,6 +1468,18 @@ __device__ __forceinline__ void finish_call(const DedupArgs& a, uint32_t G,
   __threadfence();
 }
 
+// arrivals: the blocks that get here, at least the G that share the work (the
+// others by leave_general_to).
+__device__ __forceinline__ void finish_call(const DedupArgs& a, uint32_t G, uint32_t arrivals,
+                                            unsigned long long slots0,
+                                            unsigned long long total,
+                                            unsigned long long s_stored,
+                                            unsigned long long evict,
+                                            unsigned long long s_vbytes,
+                                            const unsigned long long* s_sum) {
+  if (last_to_arrive(a.ctl, arrivals))
+    publish_call(a, G == 1, slots0, total, s_stored, evict, s_vbytes, s_sum);
+}
 
 // The rest of a call whose every chunk is a cache hit (DevCtl::any_miss), done
 // by k_dedup after its first phase: hit masks of ones, the matched slots, and
@@ -1511,7 +1530,7 @@ __device__ __noinline__ void publish_all_hits(const DedupArgs& a, uint32_t G, ui
     }
   }
   if (tid == 0) a.ctl->published = a.seq;
-  finish_call(a, G, slots0, 0ull, 0ull, 0ull, 0ull, s_sum);
+  finish_call(a, G, G, slots0, 0ull, 0ull, 0ull, 0ull, s_sum);
 }
 
 // Second kernel of the call (a regular launch sized for the copies): hit
@@ -1521,9 +1540,10 @@ __device__ __noinline__ void publish_all_hits(const DedupArgs& a, uint32_t G, ui
 // and leaves the per-call state zeroed.  Nothing is written after an error.
 // kPlain: the misses are copied by whole warps (DedupArgs::plain_copy), a
 // variant of its own so that the bulk copies' kernels carry none of its code.
+// arrivals: as for finish_call.
 template <bool kPlain>
 __device__ __forceinline__ void pack_publish(const DedupArgs& a, uint32_t G, uint32_t bid,
-                                             uint8_t* pack_smem) {
+                                             uint8_t* pack_smem, uint32_t arrivals) {
   __shared__ unsigned long long red64[kWarps];
   __shared__ unsigned long long s_slots0, s_total, s_evict;
   // a grid of one block keeps its totals here instead of in the control block
@@ -1837,7 +1857,7 @@ __device__ __forceinline__ void pack_publish(const DedupArgs& a, uint32_t G, uin
     }
   }
 
-  finish_call(a, G, slots0, total, s_stored, evict, s_vbytes, s_sum);
+  finish_call(a, G, arrivals, slots0, total, s_stored, evict, s_vbytes, s_sum);
 }
 
 // ---- one-launch resolve + pack of a one-payload call --------------------------
@@ -1872,13 +1892,15 @@ __device__ __forceinline__ uint32_t bytes_not(uint32_t w, uint32_t v) {
 // may be two different pairs'); then the group minima are posted, and the
 // rounds, ranks and copies of k_dedup and k_pack run.  Out of line, so that
 // the common path's code stays compact (the kernel runs once per call, on SMs
-// whose instruction caches are cold).  Every thread of every block calls it;
-// mine: this thread holds a chunk of a group (entry e, group key and length).
+// whose instruction caches are cold).  Every thread of blocks 0 .. G-1 calls it,
+// the other blocks of the grid (`arrivals` in all) call leave_general_to; mine:
+// this thread holds a chunk of a group (entry e, group key and length).
 template <bool kPlain>
 __device__ __noinline__ void resolve_pack_general(const DedupArgs& a, uint32_t G, uint32_t bid,
-                                                  uint8_t* smem, bool ok, bool pre, bool mine,
-                                                  uint32_t e, unsigned long long key,
-                                                  uint32_t len, uint32_t g) {
+                                                  uint32_t arrivals, uint8_t* smem, bool ok,
+                                                  bool pre, bool mine, uint32_t e,
+                                                  unsigned long long key, uint32_t len,
+                                                  uint32_t g) {
   if (pre) {
     if (mine && e != 0xFFFFFFFFu)
       *reinterpret_cast<volatile unsigned long long*>(&a.tbl[e]) = 0ull;
@@ -1897,7 +1919,19 @@ __device__ __noinline__ void resolve_pack_general(const DedupArgs& a, uint32_t G
   ok = grid_barrier(a.ctl, G, a.wait_ns, false);
   resolve_rank(a, G, bid, true, ok);
   grid_barrier(a.ctl, G, a.wait_ns, false);
-  pack_publish<kPlain>(a, G, bid, smem);
+  pack_publish<kPlain>(a, G, bid, smem, arrivals);
+}
+
+// A block of the one-launch kernel that leaves the general algorithm to others.
+// It may start after they are through, and decides by shared_groups that it has
+// nothing to do: so it is counted at the end of the call like them, the last of
+// the whole grid publishes, and no block of the call reads a control block that
+// is already the next call's.  slots0: the slots used before the call.
+__device__ __noinline__ void leave_general_to(const DedupArgs& a, uint32_t arrivals,
+                                              unsigned long long slots0) {
+  if (!last_to_arrive(a.ctl, arrivals)) return;
+  publish_call(a, false, slots0, __ldcg(&a.ctl->acc_misses), __ldcg(&a.ctl->acc_stored),
+               __ldcg(&a.ctl->evict_k), __ldcg(&a.ctl->acc_victim_bytes), nullptr);
 }
 
 template <bool kPlain>
@@ -1979,8 +2013,8 @@ __device__ __forceinline__ void resolve_pack_fast(const DedupArgs& a, uint32_t G
   if (G == 1) ok = s_err == 0;  // a grid of one did not read the error word
 
   if (s_shared) {
-    resolve_pack_general<kPlain>(a, G, bid, smem, ok, false, valid && st != kHit0 && st != kUncached, e,
-                         key, len, g);
+    resolve_pack_general<kPlain>(a, G, bid, G, smem, ok, false,
+                                 valid && st != kHit0 && st != kUncached, e, key, len, g);
     return;
   }
 
@@ -2218,7 +2252,7 @@ __device__ __forceinline__ void resolve_pack_fast(const DedupArgs& a, uint32_t G
       if (b_spec_used) atomicAdd(&a.ctl->spec_used, b_spec_used);
     }
   }
-  finish_call(a, G, slots0, total, stotal, 0ull, 0ull, s_sum);
+  finish_call(a, G, G, slots0, total, stotal, 0ull, 0ull, s_sum);
 }
 
 // The one-launch path where the hash kernel has claimed the misses' groups
@@ -2342,7 +2376,10 @@ __device__ __forceinline__ void resolve_direct(const DedupArgs& a, uint32_t G, u
     // a group may be shared: the general algorithm, from cleared outputs, on the
     // first Gg blocks, each with a larger share of the chunks
     const uint32_t Gg = min(G, a.general_blocks);
-    if (bid >= Gg) return;
+    if (bid >= Gg) {
+      leave_general_to(a, G, slots0);
+      return;
+    }
     const uint32_t pg = (N + Gg - 1) / Gg;  // <= kThreads, too
     const uint32_t c = bid * pg + threadIdx.x;
     const bool mine = threadIdx.x < pg && c < N;
@@ -2354,7 +2391,7 @@ __device__ __forceinline__ void resolve_direct(const DedupArgs& a, uint32_t G, u
     }
     const bool grouped = mine && (sh.bits[c >> 5] >> (c & 31) & 1u);
     if (mine && !grouped) ch.res[c] = kResHit0;
-    resolve_pack_general<kPlain>(a, Gg, bid, smem, ok, true, grouped,
+    resolve_pack_general<kPlain>(a, Gg, bid, G, smem, ok, true, grouped,
                                  grouped ? ch.ent[c] : 0xFFFFFFFFu, grouped ? ch.key[c] : 0ull,
                                  grouped ? ch.len[c] : 0u, c);
     return;
@@ -2608,7 +2645,7 @@ __global__ void GLEAM_PACK_BOUNDS k_pack(DedupArgs a) {
   pdl_trigger();
   pdl_wait();
   if (ldcg_u32(&a.ctl->published) == a.seq) return;  // a call of hits alone (publish_all_hits)
-  pack_publish<kPlain>(a, gridDim.x, blockIdx.x, pack_smem);
+  pack_publish<kPlain>(a, gridDim.x, blockIdx.x, pack_smem, gridDim.x);
 }
 
 // A whole small call in one block: the staged hash of its chunks (kThreads / 4
@@ -2627,7 +2664,7 @@ template <bool kPlain>
 __device__ __noinline__ void small_call_general(const DedupArgs& a, uint8_t* smem) {
   resolve_rank(a, 1, 0);
   __syncthreads();
-  pack_publish<kPlain>(a, 1, 0, smem);
+  pack_publish<kPlain>(a, 1, 0, smem, 1);
 }
 
 //

@@ -269,8 +269,8 @@ struct DedupArgs {
   uint32_t pre_claimed;
   uint32_t seq;              // number of the call, never 0
   // k_resolve_direct: blocks that run the general algorithm, with its grid
-  // barriers, where a group is shared (the others leave): few enough that the
-  // calls of two caches fit the GPU together
+  // barriers, where a group is shared (the others only count themselves at its
+  // end): few enough that the calls of two caches fit the GPU together
   uint32_t general_blocks;
   // one-launch resolve + pack: pieces of misses a warp takes at a time from a
   // counter of the call (1..32), or 0 for an equal share per warp

@@ -1,0 +1,37 @@
+"""Builds and loads tests/native/helper.cu (on a machine with a GPU only)."""
+from __future__ import annotations
+
+import ctypes
+import os
+import subprocess
+
+from paper_2607_23115_gb300 import binding as B
+from paper_2607_23115_gb300 import build as G
+
+SRC = os.path.join(os.path.dirname(os.path.abspath(__file__)), "native", "helper.cu")
+OUT = os.path.join(G.BUILD, "libtesthelper.so")
+_lib = None
+
+
+def helper() -> ctypes.CDLL:
+    global _lib
+    if _lib is None:
+        B.lib()
+        if not os.path.exists(OUT) or os.path.getmtime(OUT) < max(
+                os.path.getmtime(p) for p in (SRC, B.LIB_PATH)):
+            os.makedirs(G.BUILD, exist_ok=True)
+            tmp = "%s.tmp%d" % (OUT, os.getpid())
+            subprocess.check_call([G.NVCC, *G.ARCH, "-O2", "-std=c++17", "-Xcompiler", "-fPIC",
+                                   "-shared", "-I", G.INCLUDE, "-I", G.CSRC, "-o", tmp, SRC,
+                                   B.LIB_PATH])
+            os.replace(tmp, OUT)
+        _lib = ctypes.CDLL(OUT)
+    return _lib
+
+
+def hold(smem: int, ns: int, stream) -> None:
+    """A block that holds smem bytes of shared memory on every SM for ns."""
+    f = helper().helper_hold
+    f.argtypes = [ctypes.c_uint64, ctypes.c_uint64, ctypes.c_void_p]
+    rc = f(smem, ns, stream.cuda_stream)
+    assert rc == 0, rc
