@@ -1028,7 +1028,15 @@ __device__ __forceinline__ bool resolve_rank(const DedupArgs& a, uint32_t G, uin
   bool any_miss = true;
   bool ok = claimed ? ok0 : grid_barrier(a.ctl, G, a.wait_ns, skip, &any_miss);
   // nothing but cache hits: no rounds and no ranks (and no misses counted)
-  if (ok && !any_miss) return true;
+  if (ok && !any_miss) {
+    if (G > 1) return true;
+    // a grid of one did not read the error word: after an error of the hash
+    // kernel nothing is written, and k_pack gives the last uses back
+    if (threadIdx.x == 0) s_err1 = ld_volatile_s32(&a.ctl->err);
+    __syncthreads();
+    if (s_err1 == 0) return true;
+    ok = false;
+  }
 
   // ---- B/C: rounds until every chunk is a hit, duplicate or leader ---------
   uint32_t round = 1;

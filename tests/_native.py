@@ -35,3 +35,22 @@ def hold(smem: int, ns: int, stream) -> None:
     f.argtypes = [ctypes.c_uint64, ctypes.c_uint64, ctypes.c_void_p]
     rc = f(smem, ns, stream.cuda_stream)
     assert rc == 0, rc
+
+
+class HitsOut(ctypes.Structure):
+    _fields_ = [("status", ctypes.c_int64), ("hits", ctypes.c_int64), ("calls", ctypes.c_int64),
+                ("mask0", ctypes.c_uint64), ("slots_ok", ctypes.c_uint64),
+                ("uses_old", ctypes.c_uint64), ("uses_new", ctypes.c_uint64),
+                ("ctl_left", ctypes.c_uint64)]
+
+
+def all_hits(grid: int, nch: int, bar_count: int = 0, err: int = 0,
+             wait_ns: int = 4_000_000_000) -> HitsOut:
+    """A call of hits alone in an evicting cache (helper_all_hits)."""
+    f = helper().helper_all_hits
+    f.argtypes = [ctypes.c_uint32, ctypes.c_uint32, ctypes.c_uint32, ctypes.c_int,
+                  ctypes.c_uint64, ctypes.c_void_p]
+    out = HitsOut()
+    rc = f(grid, nch, bar_count, err, wait_ns, ctypes.byref(out))
+    assert rc == 0, rc
+    return out

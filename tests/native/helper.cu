@@ -2,6 +2,12 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <cstring>
+#include <vector>
+
+#include "gleam_internal.cuh"
+
+using namespace gleam;
 
 // Holds smem bytes of shared memory per block for about ns nanoseconds.
 __global__ void k_hold(unsigned long long ns) {
@@ -30,4 +36,131 @@ extern "C" int helper_hold(uint64_t smem, uint64_t ns, cudaStream_t stream) {
   if (e != cudaSuccess) return (int)e;
   k_hold<<<sms, 32, smem, stream>>>(ns);
   return (int)cudaGetLastError();
+}
+
+// Device memory that starts zeroed (or as given), freed with the object.
+template <typename T>
+struct Dev {
+  T* p = nullptr;
+  size_t n;
+  explicit Dev(size_t count, const T* from = nullptr) : n(count) {
+    if (cudaMalloc(&p, n * sizeof(T)) != cudaSuccess) p = nullptr;
+    if (from) cudaMemcpy(p, from, n * sizeof(T), cudaMemcpyHostToDevice);
+    else cudaMemset(p, 0, n * sizeof(T));
+  }
+  ~Dev() { cudaFree(p); }
+  std::vector<T> host() const {
+    std::vector<T> v(n);
+    cudaMemcpy(v.data(), p, n * sizeof(T), cudaMemcpyDeviceToHost);
+    return v;
+  }
+};
+
+// What a call of cache hits alone left behind.
+struct HitsOut {
+  int64_t status, hits, calls;
+  uint64_t mask0, slots_ok, uses_old, uses_new, ctl_left;
+};
+
+// The resolve kernel on `grid` blocks and the pack kernel on one, for nch chunks
+// that all hit (chunk g slot g, last used at 3) in an evicting cache whose clock
+// is at 9, with the control block's barrier count and error word as given.
+extern "C" int helper_all_hits(uint32_t grid, uint32_t nch, uint32_t bar_count, int err,
+                               uint64_t wait_ns, HitsOut* out) {
+  if (nch == 0 || nch > 4096 || grid == 0 || grid > 32) return (int)cudaErrorInvalidValue;
+  const uint64_t C = 1024, icap = 8192;
+  std::vector<uint32_t> len(nch, (uint32_t)C), ent(nch), use(nch, 3u);
+  std::vector<unsigned long long> key(nch, 7ull);
+  for (uint32_t g = 0; g < nch; ++g) ent[g] = g;
+  std::vector<unsigned long long> stats(ST_COUNT, 0ull);
+  stats[ST_SLOTS_USED] = nch;
+  std::vector<IndexEntry> none(icap);
+  std::memset(none.data(), 0xFF, icap * sizeof(IndexEntry));
+  std::vector<uint8_t> st(nch, kHit0);
+  DevCtl ctl0{};
+  ctl0.bar_count = bar_count;
+  ctl0.err = err;
+  gleam_result_t res0{};
+  res0.status = 77;
+  Dev<uint8_t> status(nch, st.data()), spec(nch), vflag(nch), buf(nch * C), packed(nch * C),
+      arena(nch * C);
+  Dev<unsigned long long> d_key(nch, key.data()), src(nch), hint(nch), cls(nch),
+      dstats(ST_COUNT, stats.data()), skey(nch);
+  Dev<uint32_t> d_len(nch, len.data()), pidx(nch), res(nch), d_ent(nch, ent.data()), rank(nch),
+      order(nch), srank(nch), old(nch), last(nch, use.data()), victims(nch), bins(kLruBins),
+      slen(nch, len.data()), bcount(4096), mask((nch + 31) / 32), idx(nch), slots(nch);
+  Dev<IndexEntry> index(icap, none.data()), hints(icap, none.data());
+  Dev<CallEntry> tbl(8192);
+  Dev<DevCtl> ctl(1, &ctl0);
+  Dev<gleam_result_t> total(1, &res0);
+  DedupArgs a{};
+  a.one.buf = buf.p;
+  a.one.n = nch * C;
+  a.one.nchunks = nch;
+  a.one.mask = mask.p;
+  a.one.miss_idx = idx.p;
+  a.one.packed = packed.p;
+  a.one.chunk_slot = slots.p;
+  a.count = 1;
+  a.Ntot = nch;
+  a.C = C;
+  a.arena = arena.p;
+  a.index = index.p;
+  a.hints = hints.p;
+  a.index_mask = icap - 1;
+  a.nslots = nch;
+  a.slot_len = slen.p;
+  a.slot_key = skey.p;
+  a.dstats = dstats.p;
+  a.ch.status = status.p;
+  a.ch.key = d_key.p;
+  a.ch.len = d_len.p;
+  a.ch.src = src.p;
+  a.ch.pidx = pidx.p;
+  a.ch.res = res.p;
+  a.ch.ent = d_ent.p;
+  a.ch.rank = rank.p;
+  a.ch.hint = hint.p;
+  a.ch.order = order.p;
+  a.ch.srank = srank.p;
+  a.ch.old = old.p;
+  a.ch.spec = spec.p;
+  a.ch.cls = cls.p;
+  a.tbl = tbl.p;
+  a.tbl_mask = tbl.n - 1;
+  a.bcount = bcount.p;
+  a.pstart = bcount.p + 4095;
+  a.ctl = ctl.p;
+  a.total = total.p;
+  a.ncalls = 1;
+  a.wait_ns = wait_ns;
+  a.skip_block = -1;
+  a.seq = 1;
+  a.lru = 1;
+  a.epoch = 9;
+  a.last_use = last.p;
+  a.vflag = vflag.p;
+  a.victims = victims.p;
+  a.bins = bins.p;
+  cudaError_t e = cudaDeviceSynchronize();
+  if (e == cudaSuccess) e = launch_dedup(a, (int)grid, 1, nullptr, false);
+  if (e == cudaSuccess) e = cudaDeviceSynchronize();
+  if (e != cudaSuccess) return (int)e;
+  const gleam_result_t r = total.host()[0];
+  out->status = r.status;
+  out->hits = (int64_t)r.n_hit_cache;
+  out->calls = (int64_t)dstats.host()[ST_CALLS];
+  out->mask0 = mask.host()[0];
+  out->slots_ok = out->uses_old = out->uses_new = out->ctl_left = 0;
+  const std::vector<uint32_t> sl = slots.host(), lu = last.host();
+  for (uint32_t g = 0; g < nch; ++g) {
+    out->slots_ok += sl[g] == g;
+    out->uses_old += lu[g] == 3;
+    out->uses_new += lu[g] == 9;
+  }
+  DevCtl left = ctl.host()[0];
+  left.published = 0;  // each call's first kernel sets it
+  const uint8_t* b = reinterpret_cast<const uint8_t*>(&left);
+  for (size_t k = 0; k < sizeof(DevCtl); ++k) out->ctl_left += b[k] != 0;
+  return 0;
 }
