@@ -925,9 +925,11 @@ __device__ __forceinline__ void post_minimum(const DedupArgs& a, uint32_t e, uin
 // The first-occurrence resolution and miss ranks of a call, run by block
 // `bid` of a grid of G co-resident blocks.  claimed: the caller has done
 // phase A (claims and minima posted, outputs cleared) and passed a grid
-// barrier since, with outcome `ok0`.
+// barrier since, with outcome `ok0`.  True if no chunk missed; *hits_ok then
+// tells whether the block's barrier was passed and no error recorded.
 __device__ __forceinline__ bool resolve_rank(const DedupArgs& a, uint32_t G, uint32_t bid,
-                                             bool claimed = false, bool ok0 = true) {
+                                             bool claimed = false, bool ok0 = true,
+                                             bool* hits_ok = nullptr) {
   __shared__ unsigned long long red64[kWarps];
   __shared__ uint32_t warp_cnt[kWarps];
   __shared__ uint32_t warp_off[kWarps];
@@ -1027,15 +1029,16 @@ __device__ __forceinline__ bool resolve_rank(const DedupArgs& a, uint32_t G, uin
   }
   bool any_miss = true;
   bool ok = claimed ? ok0 : grid_barrier(a.ctl, G, a.wait_ns, skip, &any_miss);
-  // nothing but cache hits: no rounds and no ranks (and no misses counted)
-  if (ok && !any_miss) {
-    if (G > 1) return true;
-    // a grid of one did not read the error word: after an error of the hash
-    // kernel nothing is written, and k_pack gives the last uses back
-    if (threadIdx.x == 0) s_err1 = ld_volatile_s32(&a.ctl->err);
-    __syncthreads();
-    if (s_err1 == 0) return true;
-    ok = false;
+  // nothing but cache hits, as far as a block whose wait ran out can know: no
+  // rounds and no ranks (and no misses counted)
+  if (!any_miss) {
+    if (G == 1) {  // its barrier did not read the error word
+      if (threadIdx.x == 0) s_err1 = ld_volatile_s32(&a.ctl->err);
+      __syncthreads();
+      ok = ok && s_err1 == 0;
+    }
+    if (hits_ok) *hits_ok = ok;
+    return true;
   }
 
   // ---- B/C: rounds until every chunk is a hit, duplicate or leader ---------
@@ -1367,9 +1370,9 @@ __device__ __noinline__ void clear_after_error(const DedupArgs& a) {
 // bytes, stored bytes, chunks written ahead, of them used), else the control
 // block's.
 //
-// Whether the calling block is the last of n to get here; what the others wrote
-// before is then visible to it.  Called by every thread.
-__device__ __forceinline__ bool last_to_arrive(DevCtl* ctl, uint32_t n) {
+// Whether the calling block is the last of n to count itself here; what the
+// others wrote before is then visible to it.  Called by every thread.
+__device__ __forceinline__ bool last_to_arrive(unsigned int* count, uint32_t n) {
   __shared__ int s_last;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -1377,7 +1380,7 @@ __device__ __forceinline__ bool last_to_arrive(DevCtl* ctl, uint32_t n) {
       s_last = 1;
     } else {
       __threadfence();
-      s_last = atomicAdd(&ctl->done, 1u) == n - 1;
+      s_last = atomicAdd(count, 1u) == n - 1;
     }
   }
   __syncthreads();
@@ -1465,6 +1468,7 @@ __device__ __forceinline__ void publish_call(const DedupArgs& a, bool one,
     c->unres[0] = c->unres[1] = c->unres[2] = 0;
     c->shared_groups = 0;
     c->any_miss = 0;
+    c->hits_done = 0;
     c->acc_hits_cache = c->acc_hits_intra = c->acc_rejects = 0;
     c->acc_misses = c->acc_miss_bytes = 0;
     c->acc_stored = c->acc_stored_bytes = 0;
@@ -1485,7 +1489,7 @@ __device__ __forceinline__ void finish_call(const DedupArgs& a, uint32_t G, uint
                                             unsigned long long evict,
                                             unsigned long long s_vbytes,
                                             const unsigned long long* s_sum) {
-  if (last_to_arrive(a.ctl, arrivals))
+  if (last_to_arrive(&a.ctl->done, arrivals))
     publish_call(a, G == 1, slots0, total, s_stored, evict, s_vbytes, s_sum);
 }
 
@@ -1497,7 +1501,13 @@ __device__ __forceinline__ void finish_call(const DedupArgs& a, uint32_t G, uint
 // call without it, 183 with.  Had the hash kernel stored the flag, once per
 // warp that held a miss, k_dedup could leave its first phase too (181 us), but
 // the stores to one address cost 256 MiB of 1 KiB chunks 5%.  Out of line.
-__device__ __noinline__ void publish_all_hits(const DedupArgs& a, uint32_t G, uint32_t bid) {
+//
+// ok: the block passed its barrier and saw no error.  The blocks need not agree on
+// that (a wait may run out as the last block arrives), so each is counted
+// whatever it saw, and the last of them decides by the error word: after an
+// error the call stays unpublished, and k_pack ends it as it ends any failed one.
+__device__ __noinline__ void publish_all_hits(const DedupArgs& a, uint32_t G, uint32_t bid,
+                                              bool ok) {
   __shared__ unsigned long long red64[kWarps];
   __shared__ unsigned long long s_sum[7];
   const uint32_t N = (uint32_t)a.Ntot;
@@ -1505,7 +1515,7 @@ __device__ __noinline__ void publish_all_hits(const DedupArgs& a, uint32_t G, ui
   const ChunkArrays& ch = a.ch;
   const unsigned long long slots0 =
       *(volatile const unsigned long long*)&a.dstats[ST_SLOTS_USED];
-  for (uint32_t p = tid; p < a.count; p += nth) {
+  for (uint32_t p = ok ? tid : a.count; p < a.count; p += nth) {
     const PayloadDesc& P = desc(a, p);
     gleam_result_t* r = P.result;
     if (!r) continue;
@@ -1517,7 +1527,7 @@ __device__ __noinline__ void publish_all_hits(const DedupArgs& a, uint32_t G, ui
   }
   uint32_t n_spec = 0;
 #pragma unroll 4
-  for (uint32_t g = tid; g < N; g += nth) {
+  for (uint32_t g = ok ? tid : N; g < N; g += nth) {
     const PayloadDesc& P = desc(a, ch.pidx[g]);
     const unsigned long long i = g - P.chunk_base, left = P.nchunks - i;
     if ((i & 31) == 0)
@@ -1537,8 +1547,10 @@ __device__ __noinline__ void publish_all_hits(const DedupArgs& a, uint32_t G, ui
       if (b_spec) atomicAdd(&a.ctl->spec_tried, b_spec);
     }
   }
-  if (tid == 0) a.ctl->published = a.seq;
-  finish_call(a, G, G, slots0, 0ull, 0ull, 0ull, 0ull, s_sum);
+  if (!last_to_arrive(&a.ctl->hits_done, G) || !ok || ld_volatile_s32(&a.ctl->err) != 0) return;
+  __syncthreads();  // every thread has read the error word, which publish_call resets
+  if (threadIdx.x == 0) a.ctl->published = 1u;
+  publish_call(a, G == 1, slots0, 0ull, 0ull, 0ull, 0ull, s_sum);
 }
 
 // Second kernel of the call (a regular launch sized for the copies): hit
@@ -1937,7 +1949,7 @@ __device__ __noinline__ void resolve_pack_general(const DedupArgs& a, uint32_t G
 // is already the next call's.  slots0: the slots used before the call.
 __device__ __noinline__ void leave_general_to(const DedupArgs& a, uint32_t arrivals,
                                               unsigned long long slots0) {
-  if (!last_to_arrive(a.ctl, arrivals)) return;
+  if (!last_to_arrive(&a.ctl->done, arrivals)) return;
   publish_call(a, false, slots0, __ldcg(&a.ctl->acc_misses), __ldcg(&a.ctl->acc_stored),
                __ldcg(&a.ctl->evict_k), __ldcg(&a.ctl->acc_victim_bytes), nullptr);
 }
@@ -2644,7 +2656,11 @@ __global__ void __launch_bounds__(kThreads) k_resolve_pack(DedupArgs a) {
 __global__ void __launch_bounds__(kThreads, GLEAM_DEDUP_MINBLOCKS) k_dedup(DedupArgs a) {
   pdl_trigger();
   pdl_wait();
-  if (resolve_rank(a, gridDim.x, blockIdx.x)) publish_all_hits(a, gridDim.x, blockIdx.x);
+  // k_pack's question, answered anew in every call
+  if (blockIdx.x == 0 && threadIdx.x == 0) a.ctl->published = 0u;
+  bool ok = true;
+  if (resolve_rank(a, gridDim.x, blockIdx.x, false, true, &ok))
+    publish_all_hits(a, gridDim.x, blockIdx.x, ok);
 }
 
 template <bool kPlain>
@@ -2652,7 +2668,7 @@ __global__ void GLEAM_PACK_BOUNDS k_pack(DedupArgs a) {
   extern __shared__ __align__(128) uint8_t pack_smem[];
   pdl_trigger();
   pdl_wait();
-  if (ldcg_u32(&a.ctl->published) == a.seq) return;  // a call of hits alone (publish_all_hits)
+  if (ldcg_u32(&a.ctl->published)) return;  // a call of hits alone (publish_all_hits)
   pack_publish<kPlain>(a, gridDim.x, blockIdx.x, pack_smem, gridDim.x);
 }
 

@@ -82,8 +82,6 @@ struct gleam_cache {
   uint32_t* spec_mirror = nullptr;  // page-locked, mapped: [0] as of the last finished call
   int spec_hook = 0;                // GLEAM_DEBUG_SPECULATE: 0 auto, 1 always, 2 never
 
-  uint32_t seq = 0;                 // number of the latest call (DedupArgs::seq)
-
   unsigned long long wait_ns = kDefaultWaitNs;
   int skip_block = -1;
 
@@ -506,12 +504,6 @@ bool small_call(const gleam_cache* c, uint64_t Ntot, uint64_t nbytes, int skip_b
          (!(c->flags & GLEAM_EVICT_LRU) || c->slots_bound + Ntot <= c->nslots);
 }
 
-// The next call's number; 0 is no call's.
-uint32_t next_seq(gleam_cache* c) {
-  if (++c->seq == 0) ++c->seq;
-  return c->seq;
-}
-
 // After a call is enqueued: it stores at most Ntot new slots.
 void note_call(gleam_cache* c, uint64_t Ntot) {
   c->slots_bound = std::min<uint64_t>(c->nslots, c->slots_bound + Ntot);
@@ -751,7 +743,6 @@ int enqueue(gleam_cache* c, const gleam_payload_t* payloads, uint64_t count,
   d.total = d_total ? d_total : own_total ? own_total : c->d_result;
   d.ncalls = ncalls;
   d.wait_ns = c->wait_ns;
-  d.seq = next_seq(c);
   set_lru(c, &d, Ntot);
   d.skip_block = c->skip_block;
   c->skip_block = -1;  // the hook applies to one call
@@ -1573,7 +1564,6 @@ extern "C" int gleam_dedup_copy_noalloc(gleam_cache_t* c, const void* d_buf, siz
   d.total = total;
   d.ncalls = 1;
   d.wait_ns = c->wait_ns;
-  d.seq = next_seq(c);
   const bool packed_aligned = reinterpret_cast<uintptr_t>(one.packed) % 16 == 0;
   d.far = chk.saw_managed() ? 1u : 0u;
   h.far = d.far;

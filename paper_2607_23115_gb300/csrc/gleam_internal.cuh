@@ -97,7 +97,8 @@ struct DevCtl {
   // Away from bar_count, which every block polls: next to it, the blocks' stores
   // of any_miss before they arrive at the barrier made k_dedup 10% slower.
   unsigned int any_miss;   // k_dedup found a chunk that is not a cache hit
-  unsigned int published;  // DedupArgs::seq of the last call that k_dedup published itself
+  unsigned int hits_done;  // blocks of k_dedup through with a call of hits alone
+  unsigned int published;  // k_dedup published the call itself (it sets this in every call)
 };
 
 // Position of a key in a power-of-two table: the 64-bit finaliser of
@@ -267,7 +268,6 @@ struct DedupArgs {
   uint32_t* spec_mirror;
   // the hash kernel claimed the misses' groups (HashArgs::claim_tbl)
   uint32_t pre_claimed;
-  uint32_t seq;              // number of the call, never 0
   // k_resolve_direct: blocks that run the general algorithm, with its grid
   // barriers, where a group is shared (the others only count themselves at its
   // end): few enough that the calls of two caches fit the GPU together

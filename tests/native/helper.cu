@@ -135,7 +135,6 @@ extern "C" int helper_all_hits(uint32_t grid, uint32_t nch, uint32_t bar_count, 
   a.ncalls = 1;
   a.wait_ns = wait_ns;
   a.skip_block = -1;
-  a.seq = 1;
   a.lru = 1;
   a.epoch = 9;
   a.last_use = last.p;

@@ -29,3 +29,14 @@ def test_an_error_of_the_hash_kernel(grid, nch):
     o = _native.all_hits(grid, nch, err=B.GLEAM_ERR_INTERNAL)
     assert (o.status, o.hits, o.calls) == (B.GLEAM_ERR_INTERNAL, 0, 0)
     assert o.uses_old == nch and o.mask0 == 0 and o.ctl_left == 0
+
+
+@pytest.mark.parametrize("grid,arrived", [(2, 1), (7, 1), (7, 3), (7, 6), (32, 1), (32, 16)])
+def test_a_wait_that_only_some_blocks_see_run_out(grid, arrived):
+    """Blocks counted at the barrier beforehand: the first of the grid's blocks pass
+    it, the others wait until their limit.  The call fails as a whole."""
+    torch.cuda.synchronize()
+    for _ in range(20):  # which blocks pass differs
+        o = _native.all_hits(grid, 2000, bar_count=arrived, wait_ns=1_000_000)
+        assert (o.status, o.hits, o.calls) == (B.GLEAM_ERR_TIMEOUT, 0, 0)
+        assert o.uses_old == 2000 and o.ctl_left == 0
