@@ -54,7 +54,7 @@ struct LoneShared {
   unsigned long long hinted;             // mbarrier: hint written
   unsigned long long done;               // mbarrier: the fields below written
   unsigned long long hint, hint_key;
-  uint32_t hint_slot, differs, ahead, pad;
+  uint32_t hint_slot, differs, ahead, failed;  // failed: a wait of the chunk's warp ran out
 };
 
 template <bool kProbe, uint32_t kD>
@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(32 * (1 + kLoneChunks), 2) k_hash_lone(HashArg
         if (t == 0 && speculate) give_hint(pre);
       }
     }
-    ok = __all_sync(wmask, mbar_wait(done_b, 0, a.wait_ns)) && ok;
+    ok = __all_sync(wmask, mbar_wait(done_b, 0, a.wait_ns) && !m.failed) && ok;
     if (!ok) {  // the call reports it; nothing of this chunk is used
       if (kProbe) atomicCAS(&a.ctl->err, 0, (int)GLEAM_ERR_TIMEOUT);
       acc = 0;
@@ -259,9 +259,11 @@ __global__ void __launch_bounds__(32 * (1 + kLoneChunks), 2) k_hash_lone(HashArg
   auto use = [&](uint32_t t, auto mul, auto settle, auto whole) {
     constexpr bool kMul = decltype(mul)::value, kSettle = decltype(settle)::value;
     const uint32_t b = t % kLoneProds, sb = decltype(whole)::value ? kLoneStage : sbytes(t);
-    if (kMul && t >= kLoneProds)
+    if (kMul && t >= kLoneProds) {
       ok = __all_sync(0xffffffffu,
                       mbar_wait(empty_b + 8 * b, (t / kLoneProds + 1) & 1, a.wait_ns));
+      if (!ok) return;  // the chain warp may yet read the stage: it stays, and nothing is handed over
+    }
     bool d = false;
 #pragma unroll
     for (uint32_t k = 0; k < kLoneStage; k += 512) {
@@ -385,6 +387,7 @@ __global__ void __launch_bounds__(32 * (1 + kLoneChunks), 2) k_hash_lone(HashArg
     m.hint_key = hint_key;
     m.differs = diff;
     m.ahead = ahead;
+    m.failed = !ok;
     mbar_arrive(done_b);
   }
 }

@@ -5,6 +5,8 @@ import ctypes
 import os
 import subprocess
 
+import numpy as np
+
 from paper_2607_23115_gb300 import binding as B
 from paper_2607_23115_gb300 import build as G
 
@@ -54,3 +56,17 @@ def all_hits(grid: int, nch: int, bar_count: int = 0, err: int = 0,
     rc = f(grid, nch, bar_count, err, wait_ns, ctypes.byref(out))
     assert rc == 0, rc
     return out
+
+
+def hash_alone(buf, C: int, probe: bool, wait_ns: int):
+    """(fingerprints, error recorded) of the hash kernel by itself (helper_hash)."""
+    f = helper().helper_hash
+    f.argtypes = [ctypes.c_void_p, ctypes.c_uint64, ctypes.c_uint64, ctypes.c_int,
+                  ctypes.c_uint64, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p]
+    n = buf.numel()
+    fp = np.zeros(-(-n // C), dtype=np.uint64)
+    err, lone = ctypes.c_int(), ctypes.c_int()
+    rc = f(buf.data_ptr(), n, C, int(probe), wait_ns, fp.ctypes.data, ctypes.byref(err),
+           ctypes.byref(lone))
+    assert rc == 0 and lone.value == 1, (rc, lone.value)
+    return fp, err.value

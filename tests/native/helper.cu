@@ -163,3 +163,59 @@ extern "C" int helper_all_hits(uint32_t grid, uint32_t nch, uint32_t bar_count, 
   for (size_t k = 0; k < sizeof(DevCtl); ++k) out->ctl_left += b[k] != 0;
   return 0;
 }
+
+// The hash kernel alone over n bytes of device memory in chunks of C, with every
+// wait between warps limited to wait_ns.  probe: as a dedup call on an empty
+// cache launches it (fingerprints from the chunks' records); else as
+// gleam_fingerprint does.  fp: host, one word per chunk; *err: the error recorded.
+extern "C" int helper_hash(const uint8_t* d_buf, uint64_t n, uint64_t C, int probe,
+                           uint64_t wait_ns, unsigned long long* fp, int* err, int* lone) {
+  const uint64_t N = (n + C - 1) / C, icap = 1024;
+  if (N == 0 || N > 4096) return (int)cudaErrorInvalidValue;
+  std::vector<IndexEntry> none(icap);
+  std::memset(none.data(), 0xFF, icap * sizeof(IndexEntry));
+  Dev<uint8_t> status(N), spec(N), arena(C);
+  Dev<unsigned long long> key(N), src(N), hint(N), out(N), dstats(ST_COUNT), skey(1);
+  Dev<uint32_t> len(N), pidx(N), ent(N), res(N);
+  Dev<IndexEntry> index(icap, none.data()), hints(icap, none.data());
+  Dev<DevCtl> ctl(1);
+  HashArgs h{};
+  h.one.buf = d_buf;
+  h.one.n = n;
+  h.one.nchunks = N;
+  h.count = 1;
+  h.Ntot = N;
+  h.C = C;
+  h.wait_ns = wait_ns;
+  h.ctl = ctl.p;
+  if (probe) {
+    h.index = index.p;
+    h.index_mask = icap - 1;
+    h.hints = hints.p;
+    h.arena = arena.p;
+    h.slot_key = skey.p;
+    h.dstats = dstats.p;
+    h.ch.status = status.p;
+    h.ch.key = key.p;
+    h.ch.len = len.p;
+    h.ch.src = src.p;
+    h.ch.pidx = pidx.p;
+    h.ch.res = res.p;
+    h.ch.ent = ent.p;
+    h.ch.hint = hint.p;
+    h.ch.spec = spec.p;
+    h.no_hints = 1;
+  } else {
+    h.fp_out = out.p;
+  }
+  *lone = hash_is_lone(h);
+  const bool aligned = (uintptr_t)d_buf % 16 == 0 && (N == 1 || C % 16 == 0);
+  cudaError_t e = cudaDeviceSynchronize();
+  if (e == cudaSuccess) e = launch_hash(h, aligned, nullptr, false);
+  if (e == cudaSuccess) e = cudaDeviceSynchronize();
+  if (e != cudaSuccess) return (int)e;
+  const std::vector<unsigned long long> v = probe ? key.host() : out.host();
+  std::memcpy(fp, v.data(), N * 8);
+  *err = ctl.host()[0].err;
+  return 0;
+}
