@@ -47,6 +47,17 @@ __device__ __forceinline__ unsigned long long xround(unsigned long long s, unsig
          ((unsigned long long)c << 32 | (uint32_t)wp);
 }
 
+// One of the four chains over the first `full` bytes of the chunk at p, straight
+// from memory.  Out of line: only for a fingerprint whose warps gave up waiting.
+__device__ __noinline__ unsigned long long chain_from_memory(const uint8_t* p, uint32_t full,
+                                                             uint32_t lane) {
+  unsigned long long acc = xlane_start(lane);
+#pragma unroll 1
+  for (uint32_t off = 0; off < full; off += 32)
+    acc = xstep(acc, load_word<false>(p + off + 8 * lane));
+  return acc;
+}
+
 // What the warps of a block tell each other about one chunk.
 struct LoneShared {
   unsigned long long full[kLoneProds];   // mbarriers: stage of products complete
@@ -184,9 +195,13 @@ __global__ void __launch_bounds__(32 * (1 + kLoneChunks), 2) k_hash_lone(HashArg
       }
     }
     ok = __all_sync(wmask, mbar_wait(done_b, 0, a.wait_ns) && !m.failed) && ok;
-    if (!ok) {  // the call reports it; nothing of this chunk is used
-      if (kProbe) atomicCAS(&a.ctl->err, 0, (int)GLEAM_ERR_TIMEOUT);
-      acc = 0;
+    if (!ok) {
+      if constexpr (kProbe) {  // the call reports it; nothing of this chunk is used
+        atomicCAS(&a.ctl->err, 0, (int)GLEAM_ERR_TIMEOUT);
+        acc = 0;
+      } else {  // fingerprints have no status: the chunk once more, without any wait
+        acc = chain_from_memory(p, full, lane);
+      }
     }
     ChunkEnd e;
     e.g = g, e.p = p, e.len = len, e.lane = lane, e.gbase = gbase, e.pid = pid;
