@@ -2866,6 +2866,19 @@ int dedup_blocks_per_sm() {
   return nb < GLEAM_DEDUP_BLOCKS_PER_SM ? nb : GLEAM_DEDUP_BLOCKS_PER_SM;
 }
 
+// Every kernel of this file.
+cudaError_t load_dedup_kernels() {
+  return load_kernels<
+      k_dedup, k_pack<false>, k_pack<true>, k_resolve_direct<false>, k_resolve_direct<true>,
+      k_resolve_pack<false>, k_resolve_pack<true>, k_small_call<false, false, false, false>,
+      k_small_call<false, true, false, false>, k_small_call<false, false, false, true>,
+      k_small_call<false, true, false, true>, k_small_call<false, false, true, true>,
+      k_small_call<false, true, true, true>, k_small_call<true, false, false, false>,
+      k_small_call<true, true, false, false>, k_small_call<true, false, false, true>,
+      k_small_call<true, true, false, true>, k_block_check, k_debug_insert, k_check_entries,
+      k_check_slots, k_check_publish>();
+}
+
 cudaError_t launch_dedup(const DedupArgs& a, int grid, int pack_grid, cudaStream_t s, bool pdl) {
   cudaError_t e;
   // chained, and so small that several caches' calls are resident together:

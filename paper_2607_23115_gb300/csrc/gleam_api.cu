@@ -993,6 +993,7 @@ int gleam_cache_create_ex(size_t capacity_bytes, size_t chunk_bytes, uint32_t fl
   // file's device code on the GPU, which allocates the array.
   if (rc == GLEAM_OK) rc = noalloc_scratch(&c->na_scratch);
   if (rc == GLEAM_OK) step(load_hash_kernels());
+  if (rc == GLEAM_OK) step(load_dedup_kernels());
   if (rc != GLEAM_OK) {
     destroy_cache(c);
     return rc;

@@ -292,9 +292,12 @@ cudaError_t launch_hash(const HashArgs& a, bool aligned, cudaStream_t s, bool pd
 bool hash_is_staged(const HashArgs& a);
 // Whether it runs the one with a warp per chunk.
 bool hash_is_lone(const HashArgs& a);
-// Loads the hash kernels' device code on the current GPU (cache creation does
-// it, so that no later call loads code, which allocates device memory).
+// Load the device code of every kernel of hash_probe.cu / dedup_compact.cu on the
+// current GPU.  Cache creation does it, for each cache and so on each GPU: the
+// runtime loads a kernel on its first use there, which may allocate device memory
+// and waits for the kernels that are running.
 cudaError_t load_hash_kernels();
+cudaError_t load_dedup_kernels();
 // The resolve/rank kernel on `grid` blocks, then the pack kernel (masks, indices,
 // copies, inserts, publish) on `pack_grid` blocks.  pdl: both launched with
 // programmatic stream serialization if the grid is at most kRegularDedupBlocks,
@@ -553,6 +556,15 @@ __device__ __forceinline__ uint32_t block_find_payload(const PayloadDesc* table,
   if (lo == 31 && p0 + 32 < count && __ldg(&table[p0 + 32].chunk_base) <= g)
     return find_payload_in(table, p0 + 32, count, g);
   return p0 + lo;
+}
+
+// Loads these kernels on the current GPU (the query needs them there).
+template <auto... kKerns>
+cudaError_t load_kernels() {
+  cudaFuncAttributes fa;
+  cudaError_t e = cudaSuccess;
+  ((e = e == cudaSuccess ? cudaFuncGetAttributes(&fa, kKerns) : e), ...);
+  return e;
 }
 
 // Launches kern<<<grid, block, smem, s>>>(args...), with programmatic stream

@@ -468,11 +468,24 @@ Md5Table md5_table() {
 
 }  // namespace
 
-// Loads this file's kernels on the current device (a query of one of them
-// loads the module that holds them all, when the runtime loads modules lazily).
+// Every variant that launch_hash may launch.
 cudaError_t load_hash_kernels() {
-  cudaFuncAttributes fa;
-  return cudaFuncGetAttributes(&fa, k_hash_probe_staged<true, false, true>);
+  return load_kernels<
+      k_hash_lone<false, 4>, k_hash_lone<false, 6>, k_hash_lone<false, 8>, k_hash_lone<true, 4>,
+      k_hash_lone<true, 6>, k_hash_lone<true, 8>,
+      k_hash_probe_staged<false, false, false>,
+      k_hash_probe_staged<false, false, false, false, kStage, true>,
+      k_hash_probe_staged<true, false, false>, k_hash_probe_staged<true, true, false>,
+      k_hash_probe_staged<true, false, true>, k_hash_probe_staged<true, true, true>,
+      k_hash_probe_staged<true, false, true, true>, k_hash_probe_staged<true, true, true, true>,
+      k_hash_probe_staged<true, false, false, false, kStage, true>,
+      k_hash_probe_staged<true, false, true, false, kStage, true>,
+      k_hash_probe_staged<true, false, true, true, kStage, true>,
+      k_hash_probe_staged<true, false, false, false, kBigStage>,
+      k_hash_probe_staged<true, true, false, false, kBigStage>,
+      k_hash_probe_staged<true, false, true, false, kBigStage>,
+      k_hash_probe_staged<true, true, true, false, kBigStage>, k_probe_paper,
+      k_probe_paper_staged>();
 }
 
 bool hash_is_lone(const HashArgs& a) {

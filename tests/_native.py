@@ -32,7 +32,7 @@ def helper() -> ctypes.CDLL:
 
 
 def hold(smem: int, ns: int, stream) -> None:
-    """A block that holds smem bytes of shared memory on every SM for ns."""
+    """A block that holds smem bytes of shared memory for ns, on every SM if two do not fit one."""
     f = helper().helper_hold
     f.argtypes = [ctypes.c_uint64, ctypes.c_uint64, ctypes.c_void_p]
     rc = f(smem, ns, stream.cuda_stream)

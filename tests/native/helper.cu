@@ -21,12 +21,14 @@ __global__ void k_hold(unsigned long long ns) {
   } while (t - t0 < ns);
 }
 
-// One block of k_hold per SM (two do not fit) on the stream; 0 or a CUDA error.
+// k_hold on the stream: a block on every SM where two of them do not fit (more
+// than 114 KiB each), else one block.  0 or a CUDA error.
 extern "C" int helper_hold(uint64_t smem, uint64_t ns, cudaStream_t stream) {
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess && (smem <= 114 * 1024 || ns > 1000000000ull)) e = cudaErrorInvalidValue;
+  if (e == cudaSuccess && (smem == 0 || smem > 227 * 1024 || ns > 1000000000ull))
+    e = cudaErrorInvalidValue;
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_hold, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   // the whole of the SM's shared memory, so that other kernels' blocks fit beside it
@@ -34,7 +36,7 @@ extern "C" int helper_hold(uint64_t smem, uint64_t ns, cudaStream_t stream) {
     e = cudaFuncSetAttribute(k_hold, cudaFuncAttributePreferredSharedMemoryCarveout,
                              cudaSharedmemCarveoutMaxShared);
   if (e != cudaSuccess) return (int)e;
-  k_hold<<<sms, 32, smem, stream>>>(ns);
+  k_hold<<<smem > 114 * 1024 ? sms : 1, 32, smem, stream>>>(ns);
   return (int)cudaGetLastError();
 }
 

@@ -1,0 +1,19 @@
+"""No call loads device code: cache creation has loaded every kernel."""
+import os
+import subprocess
+import sys
+
+import pytest
+
+from tests import _native
+
+pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+def test_no_call_waits_for_a_kernel_that_runs_elsewhere():
+    _native.helper()  # built before the process below needs it
+    r = subprocess.run([sys.executable, "-m", "tests._code_loading"], cwd=ROOT,
+                       stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True, timeout=300)
+    assert r.returncode == 0, r.stdout
+    assert r.stdout.strip().splitlines()[-1] == "routes 30, late: none", r.stdout
