@@ -38,7 +38,6 @@
 // grid of one block (every grid barrier a block barrier), so that the call
 // costs one launch and no kernel boundary.
 #include <algorithm>
-#include <atomic>
 
 #include "gleam_internal.cuh"
 #include "staged_hash.cuh"
@@ -2832,20 +2831,18 @@ int dedup_chunks_per_block() { return GLEAM_DEDUP_CHUNKS_PER_BLOCK; }
 // copies' buffers.
 constexpr uint32_t pack_smem_bytes(bool plain) { return plain ? 0u : kPackSmem; }
 
-// Co-resident blocks per SM of a kernel (0: unknown), asked for once (the
-// pool's GPUs are all alike): a query costs tens of microseconds of every cache
-// creation.
+// Co-resident blocks per SM of a kernel (0: unknown).
 template <auto kKern>
 int blocks_per_sm(uint32_t smem) {
-  static std::atomic<int> known{0};
-  int nb = known.load();
-  if (nb > 0) return nb;
-  if (cudaFuncSetAttribute((const void*)kKern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
-          cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kKern, kThreads, smem) != cudaSuccess)
-    return 0;
-  known.store(nb);
-  return nb;
+  static PerDevice blocks;
+  return blocks.get([smem](int) {
+    int nb = 0;
+    if (cudaFuncSetAttribute((const void*)kKern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kKern, kThreads, smem) != cudaSuccess)
+      return 0;
+    return nb;
+  });
 }
 
 // Co-resident blocks per SM of the pack kernel.

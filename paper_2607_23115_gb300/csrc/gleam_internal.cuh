@@ -1,6 +1,7 @@
 // Internal types and device helpers of libgleam (not part of the C ABI).
 #pragma once
 
+#include <atomic>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -557,6 +558,34 @@ __device__ __forceinline__ uint32_t block_find_payload(const PayloadDesc* table,
     return find_payload_in(table, p0 + 32, count, g);
   return p0 + lo;
 }
+
+// A positive figure of the current GPU, asked for once per GPU (a query costs
+// tens of microseconds); 0 if it cannot be had.
+class PerDevice {
+ public:
+  template <typename Ask>
+  int get(Ask ask) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) {
+      cudaGetLastError();
+      return 0;
+    }
+    const bool kept = dev >= 0 && dev < kDevices;
+    int v = kept ? known_[dev].load(std::memory_order_relaxed) : 0;
+    if (v > 0) return v;
+    v = ask(dev);
+    if (v <= 0) {
+      cudaGetLastError();
+      return 0;
+    }
+    if (kept) known_[dev].store(v, std::memory_order_relaxed);
+    return v;
+  }
+
+ private:
+  static constexpr int kDevices = 64;
+  std::atomic<int> known_[kDevices] = {};
+};
 
 // Loads these kernels on the current GPU (the query needs them there).
 template <auto... kKerns>

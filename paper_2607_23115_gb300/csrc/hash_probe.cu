@@ -47,26 +47,22 @@ __global__ void __launch_bounds__(kStagedThreads) k_hash_probe_staged(HashArgs a
 }
 
 // Blocks of the kS-stage variant resident at once on the whole GPU (0 if
-// unknown); cached per instantiation (the machine's GPUs are all alike).
+// unknown).
 template <bool kProbe, bool kAhead, bool kVerify, int kS>
 int staged_wave_blocks() {
-  static int wave = -1;
-  if (wave < 0) {
+  static PerDevice wave;
+  return wave.get([](int dev) {
     constexpr int smem = (kStagedThreads / 4) * group_bytes(kVerify, kS);
-    int dev = 0, nsm = 0, occ = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+    int nsm = 0, occ = 0;
+    if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
         cudaFuncSetAttribute((const void*)k_hash_probe_staged<kProbe, kAhead, kVerify, false, kS>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(
             &occ, k_hash_probe_staged<kProbe, kAhead, kVerify, false, kS>, kStagedThreads, smem) !=
-            cudaSuccess) {
-      cudaGetLastError();
+            cudaSuccess)
       return 0;
-    }
-    wave = nsm * occ;
-  }
-  return wave;
+    return nsm * occ;
+  });
 }
 
 template <bool kProbe, bool kAhead, bool kVerify, bool kPrefixAsync = false, int kS = kStage,
@@ -392,19 +388,13 @@ __global__ void __launch_bounds__(kStagedThreads) k_probe_paper_staged(HashArgs 
   }
 }
 
-// SMs of the GPU (the machine's GPUs are all alike); 0 if unknown.
+// SMs of the current GPU; 0 if unknown.
 int sm_count() {
-  static int n = -1;
-  if (n < 0) {
-    int dev = 0, v = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-      cudaGetLastError();
-      return 0;
-    }
-    n = v;
-  }
-  return n;
+  static PerDevice sms;
+  return sms.get([](int dev) {
+    int v = 0;
+    return cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess ? v : 0;
+  });
 }
 
 // Whether a call hashes with a warp per chunk (k_hash_lone) instead of the

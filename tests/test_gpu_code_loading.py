@@ -1,4 +1,5 @@
-"""No call loads device code: cache creation has loaded every kernel."""
+"""What is done once per GPU: no call loads device code, since cache creation has
+loaded every kernel, and figures of a GPU are kept for that GPU."""
 import os
 import subprocess
 import sys
@@ -17,3 +18,7 @@ def test_no_call_waits_for_a_kernel_that_runs_elsewhere():
                        stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True, timeout=300)
     assert r.returncode == 0, r.stdout
     assert r.stdout.strip().splitlines()[-1] == "routes 30, late: none", r.stdout
+
+
+def test_a_figure_is_kept_once_it_is_known():
+    assert _native.helper().helper_per_device() == 55
