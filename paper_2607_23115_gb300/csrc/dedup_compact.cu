@@ -1479,16 +1479,16 @@ __device__ __forceinline__ void publish_call(const DedupArgs& a, bool one,
   __threadfence();
 }
 
-// arrivals: the blocks that get here, at least the G that share the work (the
-// others by leave_general_to).
-__device__ __forceinline__ void finish_call(const DedupArgs& a, uint32_t G, uint32_t arrivals,
+// Every block of the grid is counted, not only the G that share the work (the
+// others get there by leave_general_to; where G is 1, so is the grid).
+__device__ __forceinline__ void finish_call(const DedupArgs& a, uint32_t G,
                                             unsigned long long slots0,
                                             unsigned long long total,
                                             unsigned long long s_stored,
                                             unsigned long long evict,
                                             unsigned long long s_vbytes,
                                             const unsigned long long* s_sum) {
-  if (last_to_arrive(&a.ctl->done, arrivals))
+  if (last_to_arrive(&a.ctl->done, G == 1 ? 1u : gridDim.x))
     publish_call(a, G == 1, slots0, total, s_stored, evict, s_vbytes, s_sum);
 }
 
@@ -1559,10 +1559,9 @@ __device__ __noinline__ void publish_all_hits(const DedupArgs& a, uint32_t G, ui
 // and leaves the per-call state zeroed.  Nothing is written after an error.
 // kPlain: the misses are copied by whole warps (DedupArgs::plain_copy), a
 // variant of its own so that the bulk copies' kernels carry none of its code.
-// arrivals: as for finish_call.
 template <bool kPlain>
 __device__ __forceinline__ void pack_publish(const DedupArgs& a, uint32_t G, uint32_t bid,
-                                             uint8_t* pack_smem, uint32_t arrivals) {
+                                             uint8_t* pack_smem) {
   __shared__ unsigned long long red64[kWarps];
   __shared__ unsigned long long s_slots0, s_total, s_evict;
   // a grid of one block keeps its totals here instead of in the control block
@@ -1876,7 +1875,7 @@ __device__ __forceinline__ void pack_publish(const DedupArgs& a, uint32_t G, uin
     }
   }
 
-  finish_call(a, G, arrivals, slots0, total, s_stored, evict, s_vbytes, s_sum);
+  finish_call(a, G, slots0, total, s_stored, evict, s_vbytes, s_sum);
 }
 
 // ---- one-launch resolve + pack of a one-payload call --------------------------
@@ -1912,14 +1911,13 @@ __device__ __forceinline__ uint32_t bytes_not(uint32_t w, uint32_t v) {
 // rounds, ranks and copies of k_dedup and k_pack run.  Out of line, so that
 // the common path's code stays compact (the kernel runs once per call, on SMs
 // whose instruction caches are cold).  Every thread of blocks 0 .. G-1 calls it,
-// the other blocks of the grid (`arrivals` in all) call leave_general_to; mine:
-// this thread holds a chunk of a group (entry e, group key and length).
+// the other blocks of the grid call leave_general_to; mine: this thread holds a
+// chunk of a group (entry e, group key and length).
 template <bool kPlain>
 __device__ __noinline__ void resolve_pack_general(const DedupArgs& a, uint32_t G, uint32_t bid,
-                                                  uint32_t arrivals, uint8_t* smem, bool ok,
-                                                  bool pre, bool mine, uint32_t e,
-                                                  unsigned long long key, uint32_t len,
-                                                  uint32_t g) {
+                                                  uint8_t* smem, bool ok, bool pre, bool mine,
+                                                  uint32_t e, unsigned long long key,
+                                                  uint32_t len, uint32_t g) {
   if (pre) {
     if (mine && e != 0xFFFFFFFFu)
       *reinterpret_cast<volatile unsigned long long*>(&a.tbl[e]) = 0ull;
@@ -1938,19 +1936,19 @@ __device__ __noinline__ void resolve_pack_general(const DedupArgs& a, uint32_t G
   ok = grid_barrier(a.ctl, G, a.wait_ns, false);
   resolve_rank(a, G, bid, true, ok);
   grid_barrier(a.ctl, G, a.wait_ns, false);
-  pack_publish<kPlain>(a, G, bid, smem, arrivals);
+  pack_publish<kPlain>(a, G, bid, smem);
 }
 
 // A block of the one-launch kernel that leaves the general algorithm to others.
 // It may start after they are through, and decides by shared_groups that it has
 // nothing to do: so it is counted at the end of the call like them, the last of
 // the whole grid publishes, and no block of the call reads a control block that
-// is already the next call's.  slots0: the slots used before the call.
-__device__ __noinline__ void leave_general_to(const DedupArgs& a, uint32_t arrivals,
-                                              unsigned long long slots0) {
-  if (!last_to_arrive(&a.ctl->done, arrivals)) return;
-  publish_call(a, false, slots0, __ldcg(&a.ctl->acc_misses), __ldcg(&a.ctl->acc_stored),
-               __ldcg(&a.ctl->evict_k), __ldcg(&a.ctl->acc_victim_bytes), nullptr);
+// is already the next call's.
+__device__ __noinline__ void leave_general_to(const DedupArgs& a) {
+  if (!last_to_arrive(&a.ctl->done, gridDim.x)) return;
+  publish_call(a, false, __ldcg(&a.dstats[ST_SLOTS_USED]), __ldcg(&a.ctl->acc_misses),
+               __ldcg(&a.ctl->acc_stored), __ldcg(&a.ctl->evict_k),
+               __ldcg(&a.ctl->acc_victim_bytes), nullptr);
 }
 
 template <bool kPlain>
@@ -2032,7 +2030,7 @@ __device__ __forceinline__ void resolve_pack_fast(const DedupArgs& a, uint32_t G
   if (G == 1) ok = s_err == 0;  // a grid of one did not read the error word
 
   if (s_shared) {
-    resolve_pack_general<kPlain>(a, G, bid, G, smem, ok, false,
+    resolve_pack_general<kPlain>(a, G, bid, smem, ok, false,
                                  valid && st != kHit0 && st != kUncached, e, key, len, g);
     return;
   }
@@ -2271,7 +2269,7 @@ __device__ __forceinline__ void resolve_pack_fast(const DedupArgs& a, uint32_t G
       if (b_spec_used) atomicAdd(&a.ctl->spec_used, b_spec_used);
     }
   }
-  finish_call(a, G, G, slots0, total, stotal, 0ull, 0ull, s_sum);
+  finish_call(a, G, slots0, total, stotal, 0ull, 0ull, s_sum);
 }
 
 // The one-launch path where the hash kernel has claimed the misses' groups
@@ -2396,7 +2394,7 @@ __device__ __forceinline__ void resolve_direct(const DedupArgs& a, uint32_t G, u
     // first Gg blocks, each with a larger share of the chunks
     const uint32_t Gg = min(G, a.general_blocks);
     if (bid >= Gg) {
-      leave_general_to(a, G, slots0);
+      leave_general_to(a);
       return;
     }
     const uint32_t pg = (N + Gg - 1) / Gg;  // <= kThreads, too
@@ -2410,7 +2408,7 @@ __device__ __forceinline__ void resolve_direct(const DedupArgs& a, uint32_t G, u
     }
     const bool grouped = mine && (sh.bits[c >> 5] >> (c & 31) & 1u);
     if (mine && !grouped) ch.res[c] = kResHit0;
-    resolve_pack_general<kPlain>(a, Gg, bid, G, smem, ok, true, grouped,
+    resolve_pack_general<kPlain>(a, Gg, bid, smem, ok, true, grouped,
                                  grouped ? ch.ent[c] : 0xFFFFFFFFu, grouped ? ch.key[c] : 0ull,
                                  grouped ? ch.len[c] : 0u, c);
     return;
@@ -2668,7 +2666,7 @@ __global__ void GLEAM_PACK_BOUNDS k_pack(DedupArgs a) {
   pdl_trigger();
   pdl_wait();
   if (ldcg_u32(&a.ctl->published)) return;  // a call of hits alone (publish_all_hits)
-  pack_publish<kPlain>(a, gridDim.x, blockIdx.x, pack_smem, gridDim.x);
+  pack_publish<kPlain>(a, gridDim.x, blockIdx.x, pack_smem);
 }
 
 // A whole small call in one block: the staged hash of its chunks (kThreads / 4
@@ -2687,7 +2685,7 @@ template <bool kPlain>
 __device__ __noinline__ void small_call_general(const DedupArgs& a, uint8_t* smem) {
   resolve_rank(a, 1, 0);
   __syncthreads();
-  pack_publish<kPlain>(a, 1, 0, smem, 1);
+  pack_publish<kPlain>(a, 1, 0, smem);
 }
 
 //
