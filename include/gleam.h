@@ -345,10 +345,12 @@ int gleam_cache_debug_insert(gleam_cache_t* cache, uint64_t key, const void* d_b
 #define GLEAM_DEBUG_DROP_ENTRY 4
 /* what = GLEAM_DEBUG_SMALL_CALLS: the largest call, in chunks, that may run as
  * one single-block kernel instead of two or three launches (default 64; 0 turns
- * that path off).  By default calls of one payload whose chunks hash faster with
- * a warp each (4 KiB and more; 32 KiB with GLEAM_OVERLAP_CALLS) run as two
- * launches all the same; once set, the limit holds for those too.  Only the
- * speed changes: every output is the same either way. */
+ * that path off).  By default calls of long chunks, which hash faster with a warp
+ * each, take the launches all the same: in caches of chunks of 4 KiB and more
+ * batches, and single payloads with a chunk of at least 1,280 bytes; with
+ * GLEAM_OVERLAP_CALLS only single payloads with a chunk of at least 36 KiB.  Once
+ * set, the limit holds for those too.  Only the speed changes: every output is the
+ * same either way. */
 #define GLEAM_DEBUG_SMALL_CALLS 5
 /* what = GLEAM_DEBUG_SPECULATE: the write-through of likely misses.  A chunk
  * that no cached chunk begins like (no prefix-hint match) is written by the

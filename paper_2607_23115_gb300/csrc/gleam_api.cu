@@ -492,7 +492,7 @@ void set_lru(gleam_cache* c, DedupArgs* d, uint64_t nchunks) {
 // A call of at most this many payload bytes may run as the single-block kernel.
 constexpr uint64_t kSmallMaxBytes = 256ull << 10;
 
-// Whether a call runs as one single-block kernel instead of three launches:
+// Whether a call may run as one single-block kernel instead of three launches:
 // few chunks and bytes (one block then hashes them about as fast as a grid
 // does, and a grid of one drops the kernel boundaries and every grid-wide
 // round trip: a 64 KiB call takes 24 us instead of 32), 64-bit or KEY16 keys,
@@ -503,6 +503,27 @@ bool small_call(const gleam_cache* c, uint64_t Ntot, uint64_t nbytes, int skip_b
          !(c->flags & GLEAM_PAPER_IDS) && skip_block < 0 &&
          (!(c->flags & GLEAM_EVICT_LRU) || c->slots_bound + Ntot <= c->nslots);
 }
+
+// A small call hashed with a warp per chunk (k_hash_lone) is faster as chained
+// launches (two for one payload, three for a batch and for KEY16 and LRU caches)
+// than as one block, whose few warps run the chunks' chains among all else, once
+// its longest chunk is long enough.  Us per call, back to back, one block against
+// chained, payloads of hits / of misses:
+//   one payload of 1,000 bytes 9.6 / 11.8 against 11.3 / 12.5, of 1,500 10.6 / 13.2
+//   against 11.1 / 12.9, of 2,500 11.4 / 13.7 against 10.9 / 12.4, of 4 KiB 12.8 /
+//   15.2 against 11.0 / 12.5, 64 KiB 93 against 45 (hits);
+//   KEY16, 1,000 bytes 14.3 / 24.7 against 14.1 / 25.6, 2,000 15.7 / 26.5 against
+//   14.2 / 25.6; LRU 15.4 / 22.7 against 15.3 / 24.0, 16.8 / 24.4 against 15.2 /
+//   24.0; one chunk of 4 / 16 / 64 KiB, KEY16 18 / 33 / 92 against 14 / 21 / 46;
+//   batches of two payloads of 500 bytes 22.8 / 31.6 against 22.9 / 33.0, of eight
+//   31 / 34.2 against 22.4 / 34.1, of two of 1,000 bytes 22.3 / 33.8 against 22.2 /
+//   34.1, of two 4 KiB chunks 24.5 / 34.1 against 21.8 / 34.1, of four 64 KiB chunks
+//   108 / 118 against 58 / 63.
+// Calls that overlap hide each other's chains (one payload; the others keep the
+// one block): 1,000 bytes 5.4 / 9.1 against 7.1 / 8.9, 32 KiB 6.4 / 9.2 against 7.3
+// / 9.3, 40,000 bytes 7.5 / 9.3 against 7.3 / 9.3, 64 KiB 11.3 / 10.4 against 9.9 /
+// 10.0.
+constexpr uint64_t kChainFrom = 1280, kChainFromOverlap = 36ull << 10;
 
 // After a call is enqueued: it stores at most Ntot new slots.
 void note_call(gleam_cache* c, uint64_t Ntot) {
@@ -658,7 +679,7 @@ int enqueue(gleam_cache* c, const gleam_payload_t* payloads, uint64_t count,
     // the staging buffer may still feed the previous call's table copy
     if ((rc = cuda_err(cudaEventSynchronize(c->table_copied))) != GLEAM_OK) return rc;
   }
-  uint64_t Ntot = 0, ncalls = 0, nbytes = 0;
+  uint64_t Ntot = 0, ncalls = 0, nbytes = 0, longest = 0;  // longest: bytes of a chunk
   bool aligned = true, packed_aligned = true;
   for (uint64_t k = 0; k < count; ++k) {
     PayloadDesc* d = count > 1 ? &c->h_table[k] : &one;
@@ -669,6 +690,7 @@ int enqueue(gleam_cache* c, const gleam_payload_t* payloads, uint64_t count,
     if (d->n) {
       ++ncalls;
       nbytes += d->n;
+      longest = std::max<uint64_t>(longest, std::min<uint64_t>(c->C, d->n));
       aligned = aligned && (reinterpret_cast<uintptr_t>(d->buf) % 16 == 0);
       packed_aligned = packed_aligned && (reinterpret_cast<uintptr_t>(d->packed) % 16 == 0);
     }
@@ -760,18 +782,13 @@ int enqueue(gleam_cache* c, const gleam_payload_t* payloads, uint64_t count,
   h.wait_late = chain && (c->flags & GLEAM_OVERLAP_CALLS) &&
                         !(c->flags & (GLEAM_PAPER_IDS | GLEAM_EVICT_LRU))
                     ? 1u : 0u;
-  // A call hashed with a warp per chunk is faster as chained launches than as
-  // one block, whose few warps run the chunks' chains among all else.  One
-  // payload, two launches against one block: one chunk of 64 KiB 45 us against
-  // 93, of 16 KiB 21 against 31, of 4 KiB 13.4 against 14.8, 64 chunks of 4 KiB
-  // 20 against 32; batches, three launches: 4 payloads of one 64 KiB chunk 66
-  // against 117, 60 of one 4 KiB chunk 40 against 51.  (Chunks of 1 KiB keep the
-  // one block: 11.5 us against 12.5 for one, and where calls overlap chunks
-  // under 32 KiB, 5.4 against 6.7, and batches.)
+  const bool overlap = (c->flags & GLEAM_OVERLAP_CALLS) != 0;
   const bool direct = chain && count == 1 && !d.classes && !d.lru;
   const bool fused =
       small_call(c, Ntot, nbytes, d.skip_block) &&
-      (c->small_forced || !hash_is_lone(h) || !(direct || !(c->flags & GLEAM_OVERLAP_CALLS)));
+      (c->small_forced ||
+       !(hash_is_lone(h) &&
+         (overlap ? direct && longest >= kChainFromOverlap : count > 1 || longest >= kChainFrom)));
   // host payloads too: a chunk written ahead then spares the pack a second
   // read over the CPU-GPU link (managed memory stays out)
   set_spec(c, &h, &d, aligned && packed_aligned && !chk.saw_managed() && !h.wait_late);
@@ -782,7 +799,7 @@ int enqueue(gleam_cache* c, const gleam_payload_t* payloads, uint64_t count,
   if (one_launch) {
     // at most one chunk per thread, and more blocks by the payload's bytes, so
     // that the misses' copies spread
-    const bool solo = !(c->flags & GLEAM_OVERLAP_CALLS);
+    const bool solo = !overlap;
     auto blocks_of = [&](uint64_t bytes) { return (nbytes + bytes - 1) / bytes; };
     const uint64_t copy_blocks =
         solo ? blocks_of(nbytes < kSoloSmallCall ? kSmallBytesPerBlock : kSoloBytesPerBlock)
@@ -802,7 +819,7 @@ int enqueue(gleam_cache* c, const gleam_payload_t* payloads, uint64_t count,
   // kChainBytesPerBlock): its warps then share the copies out as they go
   // (Llama-3-8B, one call per tensor: +1%, four layers of it: +3%), where an
   // equal share per warp suits the one-block-per-SM grid of a call on its own
-  if (one_launch && rp_grid > 1 && (c->flags & GLEAM_OVERLAP_CALLS)) d.copy_grab = kOverlapCopyGrab;
+  if (one_launch && rp_grid > 1 && overlap) d.copy_grab = kOverlapCopyGrab;
   if (one_launch && hash_is_staged(h)) {
     h.claim_tbl = d.tbl;
     h.claim_mask = d.tbl_mask;

@@ -16,12 +16,12 @@ import pytest  # noqa: E402
 
 @pytest.fixture(params=["one-kernel", "three-kernels", "write-through"])
 def call_path(request, monkeypatch):
-    """Runs a test three times: as the library runs it (a call of at most 64
-    chunks and 256 KiB as one single-block kernel, the write-through of likely
-    misses in its automatic mode), with every call on the three-launch path
-    (hash kernel, cooperative resolve kernel, pack kernel), and with the
-    write-through on for every eligible chunk, so that each path meets every
-    parity case.  Outputs must not differ."""
+    """Runs a test three times: as the library runs it (calls of at most 64
+    chunks and 256 KiB as one single-block kernel where their chunks are short,
+    other calls of one payload as two chained launches or three; the
+    write-through of likely misses in its automatic mode), with no call on the
+    single-block kernel, and with the write-through on for every eligible chunk,
+    so that each path meets every parity case.  Outputs must not differ."""
     if request.param != "one-kernel":
         from paper_2607_23115_gb300 import binding as B
         from paper_2607_23115_gb300.cache import Cache

@@ -48,7 +48,6 @@ def test_edges_of_the_single_block_path(key16):
     C = 4 * KiB
     flags = B.GLEAM_KEY16 if key16 else 0
     # chunks and tail bytes around 64 chunks / 256 KiB; offset 4 is unaligned
-    # (always the three-launch path)
     calls = [(1, 0, 0), (0, 100, 0), (63, 0, 0), (64, 0, 0), (63, 4095, 0), (64, 1, 0),
              (65, 0, 0), (2, 0, 4), (40, 17, 0), (64, 0, 0), (16, 0, 0)]
     on = _run(64, C, flags, calls, seed=1)
@@ -101,6 +100,33 @@ def test_the_library_takes_the_single_block_path():
             phase1[limit] = ms[1] * 1e3 / 20  # us per call
     assert phase1[64] < 3.0, phase1
     assert phase1[0] > 5.0, phase1
+
+
+@pytest.mark.parametrize("C,n,flags,one_block", [
+    (4 * KiB, 100, 0, True), (64 * KiB, 1279, 0, True), (64 * KiB, 1280, 0, False),
+    (4 * KiB, 900, B.GLEAM_KEY16, True), (4 * KiB, 1500, B.GLEAM_EVICT_LRU, False),
+    (KiB, 4 * KiB, 0, True), (64 * KiB, 36 * KiB - 1, B.GLEAM_OVERLAP_CALLS, True),
+    (64 * KiB, 36 * KiB, B.GLEAM_OVERLAP_CALLS, False)])
+def test_short_payloads_take_the_single_block_path(C, n, flags, one_block):
+    # by the longest chunk of the call, whatever the cache's chunk size; seen in
+    # the profile's second phase, as above (the least of several readings)
+    gc = Cache(1024 * C, C, flags)
+    oc = oracle.OracleCache(1024 * C, C, flags & (B.GLEAM_KEY16 | B.GLEAM_EVICT_LRU))
+    host = W.random_bytes(n, seed=n)
+    buf, out = host.to("cuda"), None
+    with gc:
+        dedup_both(gc, oc, host)
+        dedup_both(gc, oc, host)
+        compare_cache(gc, oc)
+        B.gleam_cache_profile(gc.handle, True)
+        per_call = []
+        for _ in range(10):
+            for _ in range(4):
+                _, out = gc.dedup(buf, out)
+            rc, ms, calls = B.gleam_cache_profile_read(gc.handle, 2)
+            assert rc == 0 and calls == [4, 4]
+            per_call.append(ms[1] * 1e3 / 4)
+    assert (min(per_call) < 3.0) == one_block, per_call
 
 
 @pytest.mark.parametrize("C", [1 * KiB, 4 * KiB, 64 * KiB])
