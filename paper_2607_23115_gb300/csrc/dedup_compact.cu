@@ -308,9 +308,14 @@ struct PackRing {
   uint32_t issued, consumed, phase;
 };
 
+// After a wait for a piece has run out: the limit for the pieces still in flight
+// to land, however short the call's own limit.  A block that ended before them
+// would leave copies under way into shared memory that another block may own.
+constexpr unsigned long long kLandNs = 1000000000ULL;
+
 // Lane 0: the whole-16-byte part of chunks 0..m-1 of `meta`; false if a
 // piece did not arrive within limit_ns (the pieces still in flight have then
-// been waited for, again with the limit).
+// been waited for).
 __device__ bool bulk_copy_batch(const PackMeta* meta, uint32_t m, uint32_t bufs, uint32_t bars,
                                 PackRing& ring, unsigned long long limit_ns) {
   auto nbytes = [&](uint32_t j) { return meta[j].len & ~15u; };
@@ -339,7 +344,7 @@ __device__ bool bulk_copy_batch(const PackMeta* meta, uint32_t m, uint32_t bufs,
     if (!mbar_wait(bars + 8 * b, (ring.phase >> b) & 1u, limit_ns)) {
       for (uint32_t k = ring.consumed; k < ring.issued; ++k) {  // let the loads land
         const uint32_t bb = k % kPackBufs;
-        mbar_wait(bars + 8 * bb, (ring.phase >> bb) & 1u, limit_ns);
+        mbar_wait(bars + 8 * bb, (ring.phase >> bb) & 1u, max(limit_ns, kLandNs));
         ring.phase ^= 1u << bb;
       }
       ring.consumed = ring.issued;
