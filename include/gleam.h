@@ -21,7 +21,9 @@
  *    arena, index and per-call workspace, allocated on the GPU that was
  *    current when the cache was created.
  *  - Errors are negative return values (enum gleam_status).  A call that
- *    returns an error other than GLEAM_ERR_CUDA leaves the cache unchanged.
+ *    returns an error other than GLEAM_ERR_CUDA leaves the cache unchanged
+ *    (but for the evictions of a GLEAM_EVICT_LRU call that timed out after
+ *    them).
  *  - Chunk i of an n-byte payload covers bytes [i*C, min(n, (i+1)*C)); the last
  *    chunk keeps its true length, and length is part of chunk equality.
  */
@@ -87,7 +89,7 @@ enum gleam_status {
                                    of device memory per slot. */
 #define GLEAM_OVERLAP_CALLS 0x10u /* consecutive calls of the cache on one
                                    stream may overlap on the GPU: a call of up
-                                   to 8192 chunks fingerprints its payload
+                                   to 16384 chunks fingerprints its payload
                                    while the calls before it are still running
                                    and waits for them (on the GPU, by
                                    programmatic dependent launch) only before

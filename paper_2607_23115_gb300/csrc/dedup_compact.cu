@@ -1350,11 +1350,16 @@ __device__ __forceinline__ bool resolve_rank(const DedupArgs& a, uint32_t G, uin
   return false;
 }
 
-// After an error that may have stopped the leaders before they cleared their
-// entries: the whole group table (and class table), and an eviction's
-// histogram and flags.  Out of line: rare, and kept out of the code that
-// every call runs.
-__device__ __noinline__ void clear_after_error(const DedupArgs& a) {
+// After an error, by the call's last block: what the failed call may have left is
+// taken back.  Its group entries, where the error stopped the leaders before they
+// cleared them (the whole group table, and class table); an eviction's histogram
+// and flags; and, if the call failed while it copied, the last uses that its hits
+// stamped and its index entries: those of slots from slots0 on, the slots used
+// before the call (they filled free entries, so the tables are then what they
+// were; what an eviction removed stays removed).  Out of line: rare, and kept out
+// of the code that every call runs.
+__device__ __noinline__ void clear_after_error(const DedupArgs& a, int err,
+                                               unsigned long long slots0) {
   for (unsigned long long e = threadIdx.x; e <= a.tbl_mask; e += kThreads) {
     a.tbl[e].owner = 0u;
     a.tbl[e].minv = 0u;
@@ -1363,6 +1368,17 @@ __device__ __noinline__ void clear_after_error(const DedupArgs& a) {
   if (a.lru) {  // an eviction that stopped half-way may have left these set
     for (uint32_t j = threadIdx.x; j < kLruBins; j += kThreads) a.bins[j] = 0u;
     for (unsigned long long j = threadIdx.x; j < a.nslots; j += kThreads) a.vflag[j] = 0;
+  }
+  if (err == (int)GLEAM_ERR_CAPACITY) return;  // found before the copies
+  if (a.lru)
+    for (unsigned long long g = threadIdx.x; g < a.Ntot; g += kThreads)
+      if (a.ch.status[g] == kHit0 && a.ch.old[g] != a.epoch)
+        a.last_use[a.ch.ent[g]] = a.ch.old[g];
+#pragma unroll 4
+  for (unsigned long long q = threadIdx.x; q <= a.index_mask; q += kThreads) {
+    const uint32_t s1 = a.index[q].slot, s2 = a.hints[q].slot;
+    if (s1 < kTombSlot && s1 >= slots0) a.index[q].slot = kEmptySlot;
+    if (s2 < kTombSlot && s2 >= slots0) a.hints[q].slot = kEmptySlot;
   }
 }
 
@@ -1462,7 +1478,7 @@ __device__ __forceinline__ void publish_call(const DedupArgs& a, bool one,
   // Leave the per-call state as the next call expects it: the group table
   // (cleared entry by entry by the leaders, or here in full after an error
   // that may have stopped them) and the control block.
-  if (err) clear_after_error(a);
+  if (err) clear_after_error(a, err, slots0);
   __syncthreads();
   if (threadIdx.x == 0) {
     DevCtl* c = a.ctl;
@@ -1610,7 +1626,8 @@ __device__ __forceinline__ void pack_publish(const DedupArgs& a, uint32_t G, uin
     return sr < evict ? (unsigned long long)__ldcg(&a.victims[sr]) : slots0 + (sr - evict);
   };
 
-  // ---- after an error: give the hit slots their last use back (LRU) ---------
+  // ---- after an error: give the hit slots their last use back (LRU; the first
+  // hit to stamp a slot kept its old value) ------------------------------------
   if (!ok && a.lru) {
     for (unsigned long long g = (unsigned long long)bid * kThreads + threadIdx.x; g < N;
          g += (unsigned long long)G * kThreads)
@@ -2572,7 +2589,7 @@ __device__ __forceinline__ void resolve_direct(const DedupArgs& a, uint32_t G, u
   __threadfence();
   const int err = ld_volatile_s32(&a.ctl->err);
   if (err) {
-    clear_after_error(a);
+    clear_after_error(a, err, slots0);
     __syncthreads();
   }
   if (threadIdx.x == 0) {
