@@ -2295,7 +2295,8 @@ __device__ __forceinline__ void resolve_pack_fast(const DedupArgs& a, uint32_t G
 }
 
 // The one-launch path where the hash kernel has claimed the misses' groups
-// (DedupArgs::pre_claimed; every miss is then stored).  If no group is shared,
+// (DedupArgs::pre_claimed; every miss is then stored, under its 64-bit key: KEY16
+// and paper identifiers claim nothing there).  If no group is shared,
 // every chunk that is not a cache hit is a miss, so every block reads the
 // statuses of the whole call (at most 16 KiB), turns them into a bit per chunk
 // with the misses counted before each word, and knows the rank of every miss,
@@ -2448,10 +2449,10 @@ __device__ __forceinline__ void resolve_direct(const DedupArgs& a, uint32_t G, u
     const uint32_t r = miss ? sh.before[g >> 5] + __popc(sh.bits[g >> 5] & ((1u << (g & 31)) - 1u)) : 0u;
     const unsigned long long slot = slots0 + r;
     const uint32_t len = (uint32_t)min(a.C, P.n - (unsigned long long)min(g, N - 1) * a.C);
-    const bool ins_hint = miss && !a.paper && len >= kPrefixBytes;
+    const bool ins_hint = miss && len >= kPrefixBytes;
     PendingInsert pi{0ull, 0u}, ph{0ull, 0u};
     if (miss) {
-      pi = index_insert_begin(a.index, a.index_mask, index_key(a, key), (uint32_t)slot);
+      pi = index_insert_begin(a.index, a.index_mask, key, (uint32_t)slot);
       if (ins_hint) ph = index_insert_begin(a.hints, a.index_mask, hint, (uint32_t)slot);
       P.miss_idx[r] = g;
       a.slot_len[slot] = len;
@@ -2559,8 +2560,7 @@ __device__ __forceinline__ void resolve_direct(const DedupArgs& a, uint32_t G, u
     // each miss completes its inserts and frees the group entry it claimed,
     // while the last pieces' stores are still in flight
     if (miss) {
-      if (!index_insert_end(a.index, a.index_mask, index_key(a, key), (uint32_t)slot, len, pi,
-                            a.key16) ||
+      if (!index_insert_end(a.index, a.index_mask, key, (uint32_t)slot, len, pi) ||
           (ins_hint && !index_insert_end(a.hints, a.index_mask, hint, (uint32_t)slot, len, ph)))
         atomicCAS(&a.ctl->err, 0, (int)GLEAM_ERR_INTERNAL);
       if (e != 0xFFFFFFFFu) a.tbl[e] = CallEntry{0u, 0u};  // owner and the claim's tag
