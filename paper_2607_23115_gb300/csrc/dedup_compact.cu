@@ -14,7 +14,8 @@
 //   * a leader counts as a verify reject iff the cache had a key+length
 //     candidate for it, or an earlier leader of the call has its key+length.
 //
-// Two launches follow the hash kernel.  k_dedup, cooperative, with phases
+// Two launches follow the hash kernel of a batch, a large call, and a call of a
+// KEY16 or evicting cache.  k_dedup, cooperative or on few blocks, with phases
 // separated by bounded grid barriers:
 //   A  outputs are cleared; every non-resident chunk claims the entry of its
 //      (key, length) in a per-call table and posts its number as the group
@@ -31,9 +32,13 @@
 // chunk slots and per-payload counters, copies every miss by rank to the
 // packed output and its arena slot and inserts it into the index; its last
 // block publishes the counters and results and leaves the per-call state
-// zeroed for the next call.
+// zeroed for the next call.  Where no chunk missed, k_dedup publishes itself.
 //
-// A call with few chunks runs instead as one single-block kernel,
+// One launch follows it for another call of one payload that is not large:
+// k_resolve_direct (k_resolve_pack for paper identifiers), which does all of
+// that.
+//
+// A call with few, short chunks runs instead as one single-block kernel,
 // k_small_call: the staged hash, then k_dedup's and k_pack's steps with a
 // grid of one block (every grid barrier a block barrier), so that the call
 // costs one launch and no kernel boundary.
@@ -1517,10 +1522,11 @@ __device__ __forceinline__ void finish_call(const DedupArgs& a, uint32_t G,
 // by k_dedup after its first phase: hit masks of ones, the matched slots, and
 // counts that follow from the payloads' sizes, without the rounds, ranks,
 // sums and atomics of the other calls; k_pack then finds the call published
-// and returns.  498 MB of 4 KiB chunks in 148 payloads, all cached: 194 us the
-// call without it, 183 with.  Had the hash kernel stored the flag, once per
-// warp that held a miss, k_dedup could leave its first phase too (181 us), but
-// the stores to one address cost 256 MiB of 1 KiB chunks 5%.  Out of line.
+// and returns.  498 MB of 4 KiB chunks in 148 payloads, all cached: 195 us the
+// call without it, 192 with (194 and 183 while a k_dedup of this grid was
+// launched early).  Had the hash kernel stored the flag, once per warp that held
+// a miss, k_dedup could leave its first phase too (2 us less), but the stores to
+// one address cost 256 MiB of 1 KiB chunks 5%.  Out of line.
 //
 // ok: the block passed its barrier and saw no error.  The blocks need not agree on
 // that (a wait may run out as the last block arrives), so each is counted
@@ -1908,7 +1914,8 @@ __device__ __forceinline__ void pack_publish(const DedupArgs& a, uint32_t G, uin
 // length) groups as it recorded them, else (paper identifiers, and the
 // single-block small call) the steps below.  Block b owns the contiguous chunks
 // [b * per, (b + 1) * per), at most one per thread.  Phase 1 classifies them
-// and claims their groups without posting minima.  If no chunk of the call
+// and claims their groups (a claim stores the claimant as the group's minimum;
+// the group's other chunks post theirs later).  If no chunk of the call
 // found its group claimed by another (no in-call duplicate and no key
 // collision: the common case), every chunk that is not a cache hit is a miss of
 // round one (its own group's first chunk), so after one grid barrier each block
@@ -1916,8 +1923,8 @@ __device__ __forceinline__ void pack_publish(const DedupArgs& a, uint32_t G, uin
 // inserts its misses; after a second barrier every warp of the grid copies its
 // share of all misses' bytes (a block's own misses would leave the blocks that
 // hold the most of them as the call's tail).  Otherwise the general algorithm
-// takes over: the minima are posted and resolve_rank and pack_publish run on
-// the same grid.
+// takes over: the other minima are posted and resolve_rank and pack_publish run
+// on the same grid.
 
 // Bit k of the result: byte k of w (k < 4) is not v.
 __device__ __forceinline__ uint32_t bytes_not(uint32_t w, uint32_t v) {

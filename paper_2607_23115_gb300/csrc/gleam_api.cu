@@ -536,14 +536,16 @@ void note_call(gleam_cache* c, uint64_t Ntot) {
 // stream be launched as soon as all of its blocks have started, so that a
 // kernel's blocks are waiting on the GPU when the one before finishes instead
 // of being launched then.  After the hash kernel, a call of one payload runs
-// resolve, ranks, pack and publish as one launch (k_resolve_direct, one block
-// per 256 chunks or kChainBytesPerBlock of payload, at most kChainPackBlocks);
-// a batch runs the resolve kernel as a regular launch (a cooperative one is
-// never launched early) and the pack kernel; where calls overlap on at most
-// kChainDedupBlocks and kChainPackBlocks blocks: every waiting block holds its
-// SM resources.  With GLEAM_OVERLAP_CALLS the hash kernel also fingerprints
-// before it waits (HashArgs::wait_late; not for evicting caches).  The test hook
-// that makes a block skip a barrier keeps the plain launches.
+// resolve, ranks, pack and publish as one launch (k_resolve_direct; one block per
+// 256 chunks, and more by the payload's bytes, see kSoloBytesPerBlock and
+// kChainBytesPerBlock); a batch, and a call of a KEY16 or evicting cache, runs the
+// resolve kernel and the pack kernel, the first as a regular launch up to
+// kRegularDedupBlocks blocks (a cooperative one is never launched early).  Where
+// calls overlap they keep to kChainDedupBlocks and kChainPackBlocks blocks: every
+// waiting block holds its SM resources.  With GLEAM_OVERLAP_CALLS the hash kernel
+// also fingerprints before it waits (HashArgs::wait_late; not for evicting
+// caches).  The test hook that makes a block skip a barrier keeps the plain
+// launches.
 #ifndef GLEAM_CHAIN_MAX_CHUNKS
 #define GLEAM_CHAIN_MAX_CHUNKS 16384
 #endif
@@ -818,7 +820,7 @@ int enqueue(gleam_cache* c, const gleam_payload_t* payloads, uint64_t count,
   // overlapping calls give the one-launch kernel few blocks (a block per
   // kChainBytesPerBlock): its warps then share the copies out as they go
   // (Llama-3-8B, one call per tensor: +1%, four layers of it: +3%), where an
-  // equal share per warp suits the one-block-per-SM grid of a call on its own
+  // equal share per warp suits the grid of a call on its own
   if (one_launch && rp_grid > 1 && overlap) d.copy_grab = kOverlapCopyGrab;
   if (one_launch && hash_is_staged(h)) {
     h.claim_tbl = d.tbl;

@@ -13,7 +13,8 @@
 // candidate is compared by re-reading both copies.
 //
 // Kernels: k_hash_probe_staged (chunks stream through shared memory by
-// cp.async; a variant for payloads of any alignment), and for the paper's
+// cp.async; a variant for payloads of any alignment), k_hash_lone (few chunks: a
+// warp for each, see lone_hash.cuh), and for the paper's
 // identifiers k_probe_paper_staged / k_probe_paper (MD5 of the first 128 bytes
 // as the key; 16-byte-aligned payloads / any alignment, by direct loads).
 #include <algorithm>
