@@ -70,7 +70,7 @@ def test_beside_a_kernel_that_leaves_room_for_one_block_per_sm(nch, flags):
             torch.cuda.synchronize()
             for k in range(len(side.calls)):
                 if beside:
-                    _native.hold(130 * KiB, 50_000_000, other)
+                    _native.hold(130 * KiB, 150_000_000, other)
                     held = other.record_event()
                 side.enqueue(k, mine)
                 mine.synchronize()
